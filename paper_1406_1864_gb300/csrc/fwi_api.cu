@@ -12,6 +12,7 @@
 // device and is queued on the caller's stream.
 #include "fwi.h"
 #include "fwi_internal.h"
+#include "fwi_resident.h"
 
 #include <cudaTypedefs.h>
 
@@ -96,6 +97,10 @@ struct Plan {
     Tiling tr{};          // tiling of the segment re-propagation (plain forward)
     Part snaps, snap_max; // [nck][2][ns][fstride] F32 / 16-bit, [nck][2][ns]
     Part seg;             // segment levels beyond the two forward buffers
+    // chip-resident time loops (ok = 0: streaming steps): the forward pass and
+    // the backward pass, and the packets their tiles exchange
+    ResTile rf{}, rb{};
+    Part xch;
     size_t total = 0;
 };
 
@@ -191,8 +196,51 @@ Lay2D make_layout(const fwi_grid *g)
     return L;
 }
 
+// whether the receivers suit a resident pass: at most RES_MAXE of a shot in one
+// tile, and (backward) those in one row
+bool receivers_fit(const Lay2D &L, const fwi_geometry *ge, const ResTile &t, bool backward)
+{
+    if (ge->nrec <= RES_MAXE && !backward) return true;
+    const size_t tiles = (size_t)t.ntx * t.ntz;
+    std::vector<int> cnt(tiles), row(tiles);
+    for (int s = 0; s < ge->nshots; ++s) {
+        std::fill(cnt.begin(), cnt.end(), 0);
+        for (int r = 0; r < ge->nrec; ++r) {
+            const int *q = ge->rec + 3 * ((long long)s * ge->nrec + r);
+            const size_t k = (size_t)((q[0] + L.P) / t.th) * t.ntx + (q[2] + L.P) / (4 * t.w4);
+            if (cnt[k]++ == 0) row[k] = q[0];
+            if (cnt[k] > RES_MAXE || (backward && row[k] != q[0])) return false;
+        }
+    }
+    return true;
+}
+
+// Level of the streaming steps in us, fitted to the measured ones (recorded
+// graphs, autotuned tiles) from 0.1 M to 34 M padded points: forward 7.1, 22.6,
+// 27.3 and 84 us at 0.13, 4.2, 7.6 and 34 M; backward 9.2, 34, 51 and 157 us.
+double streaming_us(double pts, ResKind kind)
+{
+    return kind == RES_BWD ? std::min(8.0 + 9e-6 * pts, 20.0 + 4.0e-6 * pts)
+                           : std::min(6.0 + 4.0e-6 * pts, 14.0 + 2.0e-6 * pts);
+}
+
+// The resident time loop where it is expected to be faster
+ResTile choose_resident(const Lay2D &L, int ns, ResKind kind)
+{
+    const ResTile t = res_plan(L, ns, kind);
+    return t.ok && t.us < streaming_us((double)L.nzp * L.nxp * ns, kind) ? t : ResTile{};
+}
+
+ResKind res_forward_kind(const fwi_options *o, int op)
+{
+    if (op != FWI_OP_GRADIENT && op != FWI_OP_ILLUMINATION) return RES_FWD;
+    return o->illum_mode == FWI_ILLUM_UTT2 ? RES_FWD_UTT2 : RES_FWD_U2;
+}
+
+// (allow_resident = false: streaming steps only, without the resident loops'
+// packets in the workspace)
 fwi_status make_plan(const fwi_grid *g, const fwi_geometry *ge, const fwi_options *o, int op,
-                     bool coords, Plan &pl)
+                     bool coords, Plan &pl, bool allow_resident = true)
 {
     fwi_status st;
     if ((st = check_grid(g)) != FWI_OK) return st;
@@ -200,6 +248,7 @@ fwi_status make_plan(const fwi_grid *g, const fwi_geometry *ge, const fwi_option
     if (!no_geom && (st = check_geom(g, ge, coords)) != FWI_OK) return st;
     if ((st = check_opts(o, op)) != FWI_OK) return st;
     pl.L = make_layout(g);
+    pl.rf = pl.rb = ResTile{};
     pl.op = op;
     pl.nt = g->nt;
     const Lay2D &L = pl.L;
@@ -243,6 +292,13 @@ fwi_status make_plan(const fwi_grid *g, const fwi_geometry *ge, const fwi_option
     // 2 HE + 1 image planes once)
     pl.tb = pl.ext ? make_tiling(L, pl.ns, STEP_BWD, 1, 32)
                    : (born ? make_tiling(L, pl.ns, STEP_BWD, 0) : make_tiling(L, pl.ns, STEP_BWD));
+    if (allow_resident && !pl.snap && !pl.with_offh && !(born && !need_bwd) && op != FWI_OP_GN_HVP)
+        pl.rf = choose_resident(L, pl.ns, res_forward_kind(o, op));
+    if (allow_resident && need_bwd && !pl.snap && !pl.ext) pl.rb = choose_resident(L, pl.ns, RES_BWD);
+    // (the workspace does not depend on pinned steps or the receivers' places)
+    const size_t xch = (size_t)std::max(pl.rf.xch, pl.rb.xch);
+    if (pl.rf.ok && (res_pinned(STEP_FWD, L, pl.ns) || (coords && !receivers_fit(L, ge, pl.rf, false)))) pl.rf = ResTile{};
+    if (pl.rb.ok && (res_pinned(STEP_BWD, L, pl.ns) || (coords && !receivers_fit(L, ge, pl.rb, true)))) pl.rb = ResTile{};
     const size_t fbytes = (size_t)L.fstride * sizeof(float);
     const size_t nphys = (size_t)L.nz * L.nx;
     take(pl.c2, fbytes);
@@ -305,6 +361,7 @@ fwi_status make_plan(const fwi_grid *g, const fwi_geometry *ge, const fwi_option
         tk(pl.tab_bshot, std::max<size_t>(nent, 1) * sizeof(int));
     }
     take(pl.tab, t);
+    take(pl.xch, xch);
     pl.total = off;
     return FWI_OK;
 }
@@ -315,7 +372,15 @@ template <class T> T *at(void *ws, const Part &p, size_t extra)
     return reinterpret_cast<T *>(static_cast<char *>(ws) + p.off + extra);
 }
 
-void build_csr(const Plan &pl, const Tiling &t, const int *rec, std::vector<char> &buf, size_t ptr_off,
+// tiles of a receiver table: ntx x ntz tiles of tx x tz cells
+struct TableTiles {
+    int tx, tz, ntx, ntz;
+};
+
+TableTiles table_tiles(const Tiling &t) { return {TX, t.tz, t.ntx, t.ntz}; }
+TableTiles table_tiles(const ResTile &t) { return {4 * t.w4, t.th, t.ntx, t.ntz}; }
+
+void build_csr(const Plan &pl, const TableTiles &t, const int *rec, std::vector<char> &buf, size_t ptr_off,
                size_t ent_off, size_t shot_off = (size_t)-1)
 {
     const Lay2D &L = pl.L;
@@ -326,8 +391,8 @@ void build_csr(const Plan &pl, const Tiling &t, const int *rec, std::vector<char
     auto tile_of = [&](int s, int r, int &local) {
         const int *q = rec + 3 * ((long long)s * pl.nrec + r);
         const int i = q[0] + L.P, j = q[2] + L.P;
-        const int tz = i / t.tz, tx = j / TX;
-        local = (i - tz * t.tz) * TX + (j - tx * TX);
+        const int tz = i / t.tz, tx = j / t.tx;
+        local = (i - tz * t.tz) * t.tx + (j - tx * t.tx);
         return tz * t.ntx + tx;
     };
     for (int s = 0; s < pl.ns; ++s)
@@ -360,8 +425,14 @@ fwi_status upload_tables(const Plan &pl, const fwi_geometry *ge, void *ws, cudaS
         srcij[s] = make_int2(c[0] + pl.L.P, c[2] + pl.L.P);
     }
     if (pl.nrec > 0) {
-        build_csr(pl, pl.tf, ge->rec, buf, pl.tab_fptr, pl.tab_fent);
-        if (pl.need_bwd || pl.born) build_csr(pl, pl.tb, ge->rec, buf, pl.tab_bptr, pl.tab_bent, pl.tab_bshot);
+        // forward table: of the forward pass, or of the Born pass where the
+        // backward table is a resident backward pass's
+        const bool born_f = pl.born && pl.rb.ok;
+        build_csr(pl, pl.rf.ok ? table_tiles(pl.rf) : table_tiles(born_f ? pl.tb : pl.tf), ge->rec, buf, pl.tab_fptr,
+                  pl.tab_fent);
+        if (pl.need_bwd || pl.born)
+            build_csr(pl, pl.rb.ok ? table_tiles(pl.rb) : table_tiles(pl.tb), ge->rec, buf, pl.tab_bptr, pl.tab_bent,
+                      pl.tab_bshot);
     }
     cudaError_t e = cudaMemcpyAsync(at<char>(ws, pl.tab), buf.data(), buf.size(), cudaMemcpyHostToDevice, st);
     if (e != cudaSuccess) return cuda_fail(e, "upload of geometry tables");
@@ -518,8 +589,8 @@ fwi_status run_born(const Plan &pl, const fwi_geometry *ge, void *ws, float *dse
     a.dext = he > 0 ? at<float>(ws, pl.dext) : nullptr;
     a.band = save ? at<float>(ws, pl.band) : nullptr;
     a.dseis = (dseis && pl.nrec > 0) ? dseis : nullptr;
-    a.rt.ptr = at<int>(ws, pl.tab, pl.tab_bptr);
-    a.rt.ent = at<int2>(ws, pl.tab, pl.tab_bent);
+    a.rt.ptr = at<int>(ws, pl.tab, pl.rb.ok ? pl.tab_fptr : pl.tab_bptr);
+    a.rt.ent = at<int2>(ws, pl.tab, pl.rb.ok ? pl.tab_fent : pl.tab_bent);
     float *U[2] = {at<float>(ws, pl.u[0]), at<float>(ws, pl.u[1])};
     float *DU[2] = {at<float>(ws, pl.p[0]), at<float>(ws, pl.p[1])};
     for (int b = 0; b < 2; ++b)
@@ -557,6 +628,71 @@ fwi_status run_born(const Plan &pl, const fwi_geometry *ge, void *ws, float *dse
     return FWI_OK;
 }
 
+// argument block of a resident time loop (pass 0: forward, 1: backward)
+ResArgs res_args(const Plan &pl, const fwi_geometry *ge, void *ws, int *status, int pass)
+{
+    ResArgs a{};
+    a.L = pl.L;
+    a.t = pass == 0 ? pl.rf : pl.rb;
+    a.c2 = at<float>(ws, pl.c2);
+    a.damp = at<float>(ws, pl.damp);
+    a.src_ij = at<int2>(ws, pl.tab, pl.tab_srcij);
+    a.wav = ge->wavelet;
+    a.src_scale = 1.0f; // dx^(2-ndim) in 2-D
+    a.ns = pl.ns;
+    a.nt = pl.nt;
+    a.nrec = pl.nrec;
+    a.status = status;
+    a.xch = at<uint2>(ws, pl.xch);
+    a.rptr = at<int>(ws, pl.tab, pass == 0 ? pl.tab_fptr : pl.tab_bptr);
+    a.rent = at<int2>(ws, pl.tab, pass == 0 ? pl.tab_fent : pl.tab_bent);
+    a.u[0] = at<float>(ws, pl.u[0]);
+    a.u[1] = at<float>(ws, pl.u[1]);
+    return a;
+}
+
+// the whole forward time loop of one model as one resident launch
+fwi_status run_forward_resident(const Plan &pl, const fwi_geometry *ge, void *ws, int *status, float *seis, bool save,
+                                float *acc_i, int illum_utt, cudaStream_t st)
+{
+    cudaError_t e;
+    if (acc_i && (e = cudaMemsetAsync(acc_i, 0, pl.acc_i.bytes, st)) != cudaSuccess) return cuda_fail(e, "memset");
+    ResArgs a = res_args(pl, ge, ws, status, 0);
+    a.band = save ? at<float>(ws, pl.band) : nullptr;
+    a.save = save;
+    a.seis = (seis && pl.nrec > 0) ? seis : nullptr;
+    a.acc_illum = acc_i;
+    const ResKind kind = !acc_i ? RES_FWD : (illum_utt ? RES_FWD_UTT2 : RES_FWD_U2);
+    if ((e = launch_resident(a, kind, st)) != cudaSuccess)
+        return cuda_fail(e, "resident forward loop");
+    t_launch[0]++;
+    return FWI_OK;
+}
+
+// the whole backward time loop of one model as one resident launch
+fwi_status run_backward_resident(const Plan &pl, const fwi_geometry *ge, void *ws, int *status, const float *adj,
+                                 cudaStream_t st)
+{
+    cudaError_t e;
+    if ((e = cudaMemsetAsync(at<char>(ws, pl.acc_g), 0, pl.acc_g.bytes, st)) != cudaSuccess)
+        return cuda_fail(e, "memset");
+    ResArgs a = res_args(pl, ge, ws, status, 1);
+    a.band = at<float>(ws, pl.band);
+    a.nent = pl.ns * pl.nrec;
+    if (pl.nrec > 0) {
+        if ((e = launch_permute_adj(adj, at<int2>(ws, pl.tab, pl.tab_bent), at<int>(ws, pl.tab, pl.tab_bshot), a.nent,
+                                    pl.nt, pl.nrec, at<float>(ws, pl.adj_t), st)) != cudaSuccess)
+            return cuda_fail(e, "adjoint-source permutation");
+        t_launch[2]++;
+        a.adj = at<float>(ws, pl.adj_t);
+    }
+    a.adj_scale = pl.L.dx * pl.L.dx;
+    a.acc_grad = at<float>(ws, pl.acc_g);
+    if ((e = launch_resident(a, RES_BWD, st)) != cudaSuccess) return cuda_fail(e, "resident backward loop");
+    t_launch[1]++;
+    return FWI_OK;
+}
+
 // (levels [n0, n1) only, and events around the step launches, when timing
 // tile variants)
 fwi_status run_forward_models(int nm, const Plan *pl, const fwi_geometry *const *ge, void *const *ws,
@@ -565,6 +701,14 @@ fwi_status run_forward_models(int nm, const Plan *pl, const fwi_geometry *const 
                               cudaEvent_t ev1 = nullptr)
 {
     cudaError_t e;
+    if (pl[0].rf.ok) { // every model of the call (make_batch)
+        for (int k = 0; k < nm; ++k) {
+            const fwi_status s = run_forward_resident(pl[k], ge[k], ws[k], at<int>(ws[0], pl[0].scal, 8), seis[k], save,
+                                                      acc_i[k], illum_utt, st);
+            if (s != FWI_OK) return s;
+        }
+        return FWI_OK;
+    }
     std::vector<FwdArgs> a(nm);
     std::vector<Tiling> til(nm);
     std::vector<std::array<float *, 2>> U(nm);
@@ -720,6 +864,13 @@ fwi_status run_backward_models(int nm, const Plan *pl, const fwi_geometry *const
                                float *acc_ext = nullptr)
 {
     cudaError_t e;
+    if (pl[0].rb.ok) { // every model of the call (make_batch)
+        for (int k = 0; k < nm; ++k) {
+            const fwi_status s = run_backward_resident(pl[k], ge[k], ws[k], at<int>(ws[0], pl[0].scal, 8), adj[k], st);
+            if (s != FWI_OK) return s;
+        }
+        return FWI_OK;
+    }
     std::vector<BwdArgs> a(nm);
     std::vector<Tiling> til(nm);
     std::vector<std::array<float *, 2>> U(nm), Pp(nm);
@@ -1697,6 +1848,20 @@ fwi_status make_batch(int nm, const fwi_grid *grids, const fwi_geometry *geoms, 
     for (int k = 1; k < nm; ++k)
         if ((long long)pl[k].L.nzp * pl[k].L.nxp * pl[k].ns > (long long)pl[kmax].L.nzp * pl[kmax].L.nxp * pl[kmax].ns)
             kmax = k;
+    // a pass of the batch is resident (one launch per model) where that is so
+    // for every model and expected to be faster than the batched steps
+    for (int b = 0; b < 2 && nm > 1; ++b) {
+        double pts = 0, us = 0;
+        bool all = true;
+        for (int k = 0; k < nm; ++k) {
+            const ResTile &t = b ? pl[k].rb : pl[k].rf;
+            all = all && t.ok;
+            us += t.us;
+            pts += (double)pl[k].L.nzp * pl[k].L.nxp * pl[k].ns;
+        }
+        if (all && us < streaming_us(pts, b ? RES_BWD : RES_FWD_U2)) continue;
+        for (int k = 0; k < nm; ++k) (b ? pl[k].rb : pl[k].rf) = ResTile{};
+    }
     for (int k = 0; k < nm; ++k) {
         if (k == kmax) continue;
         const StepKind fk = pl[k].with_offh ? STEP_FWD_OFFH : STEP_FWD;
@@ -2341,7 +2506,7 @@ fwi_status fwi_autotune(const fwi_grid *grid, const fwi_geometry *geom, const fw
     if (grid && grid->ndim == 3)
         return autotune3(grid, geom, opts, v, ws, ws_bytes, static_cast<cudaStream_t>(stream), choice);
     Plan pl;
-    fwi_status s = make_plan(grid, geom, opts, FWI_OP_GRADIENT, true, pl);
+    fwi_status s = make_plan(grid, geom, opts, FWI_OP_GRADIENT, true, pl, false); // the streaming steps
     if (s != FWI_OK) return s;
     if (!v) return fail(FWI_ERR_INVALID_ARG, "v is NULL");
     if ((s = check_ws(pl, ws, ws_bytes)) != FWI_OK) return s;
@@ -2411,6 +2576,7 @@ fwi_status fwi_autotune(const fwi_grid *grid, const fwi_geometry *geom, const fw
             }
         if (s != FWI_OK) break;
         step_tuned_store(kind, pl.L, pl.ns, best[kk][0], best[kk][1]);
+        res_pin(kind, pl.L, pl.ns, false);
     }
     t_prof = prof;
     if (s != FWI_OK) return s;
@@ -2455,6 +2621,8 @@ fwi_status fwi_autotune_set(const fwi_grid *grid, const fwi_geometry *geom, cons
     if (choice[1] < 1 || choice[3] < 1) return fail(FWI_ERR_INVALID_ARG, "chunk must be >= 1");
     step_tuned_store(fk, pl.L, pl.ns, choice[0], choice[1]);
     step_tuned_store(STEP_BWD, pl.L, pl.ns, choice[2], choice[3]);
+    res_pin(fk, pl.L, pl.ns, true);
+    res_pin(STEP_BWD, pl.L, pl.ns, true);
     t_err.clear();
     return FWI_OK;
 }
@@ -2462,6 +2630,7 @@ fwi_status fwi_autotune_set(const fwi_grid *grid, const fwi_geometry *geom, cons
 fwi_status fwi_autotune_reset(void)
 {
     step_tuned_clear();
+    res_pin_clear();
     step3_tuned_clear();
     return FWI_OK;
 }
@@ -2719,6 +2888,10 @@ extern "C" fwi_status fwi_forward_noalloc(const fwi_grid *grid, const fwi_geomet
     Plan pl;
     fwi_status s = make_plan(grid, geom, nullptr, FWI_OP_FORWARD, true, pl);
     if (s != FWI_OK) return s;
+    if (pl.total > (size_t)FWI_NOALLOC_SCRATCH_BYTES) { // without the resident loop's packets
+        pl = Plan{};
+        if ((s = make_plan(grid, geom, nullptr, FWI_OP_FORWARD, true, pl, false)) != FWI_OK) return s;
+    }
     if (!v || (!seis && geom->nrec > 0)) return fail(FWI_ERR_INVALID_ARG, "v or seis is NULL");
     if (pl.total > (size_t)FWI_NOALLOC_SCRATCH_BYTES)
         return fail(FWI_ERR_NOMEM,

@@ -1,0 +1,66 @@
+// fwi_resident.h -- argument block and tiling of the chip-resident 2-D time
+// loops (fwi_resident2d.cu). Not part of the public ABI.
+#pragma once
+
+#include "fwi_args.h"
+
+namespace fwi {
+
+constexpr int RES_SMAX = 8;        // most shots in flight per CTA
+constexpr int RES_SVC = 4;         // service warps per CTA
+constexpr int RES_MAXE = 256;      // most receivers of one (tile, shot)
+// forward passes without an illumination sum, with that of u^2, of u_tt^2; backward
+enum ResKind { RES_FWD = 0, RES_FWD_U2 = 1, RES_FWD_UTT2 = 2, RES_BWD = 3 };
+
+// How one pass is laid out over the chip: every shot in flight is cut into
+// ntx x ntz tiles of 4 w4 columns by th rows, one CTA each; a CTA holds its
+// tile of s shots at a time; `sets` groups of CTAs work on different shots.
+struct ResTile {
+    int ok;            // 0: the streaming steps are used
+    int variant;       // compiled (rows per thread, warps) variant of the kind
+    int w4, th, g;     // float4 columns, rows, row groups of a tile
+    int ntx, ntz;      // tiles of one shot
+    int sets, s;       // CTA groups; shots in flight per CTA
+    int per;           // shots of one set over the whole pass
+    int fs;            // floats of one field tile with its halo
+    int ne;            // float4s of a tile's edge strips
+    int smem;          // dynamic shared memory
+    long long xch;     // bytes of the exchange packets
+    float us;          // estimated time of one level of all shots, in us
+};
+
+struct ResArgs {
+    Lay2D L;
+    ResTile t;
+    const float *c2, *damp;
+    const int2 *src_ij;
+    const float *wav;      // [ns][nt]
+    float src_scale;
+    int ns, nt, nrec;
+    int *status;
+    uint2 *xch;            // packets {value, level}: [sets * s][parity][field][ntx * ntz][ne][4]
+    const int *rptr;       // receivers of (tile, shot): [ptr[t * ns + s], ptr[t * ns + s + 1])
+    const int2 *rent;      // {local = row * 4 w4 + column, r}
+    float *u[2];           // wavefields of even / odd levels, field layout
+    float *band;           // [ns][nt][nbandp]
+    // forward
+    float *seis;           // [ns][nt][nrec] or null
+    float *acc_illum;      // [nz][nx] or null
+    int save;              // the final two levels are written to u
+    // backward
+    const float *adj;      // [nt][nent], receiver-table order, or null
+    int nent;
+    float adj_scale;
+    float *acc_grad;       // [nzp][nxp]
+};
+
+// Layout of a pass over ns shots (ok = 0 where one shot does not fit the
+// chip or the streaming steps are expected to be faster)
+ResTile res_plan(const Lay2D &L, int ns, ResKind kind);
+// shapes whose streaming steps were pinned (fwi_autotune_set): no resident loop
+void res_pin(StepKind kind, const Lay2D &L, int ns, bool pinned);
+bool res_pinned(StepKind kind, const Lay2D &L, int ns);
+void res_pin_clear();
+cudaError_t launch_resident(const ResArgs &a, ResKind kind, cudaStream_t st);
+
+} // namespace fwi
