@@ -294,9 +294,11 @@ fwi_status make_plan(const fwi_grid *g, const fwi_geometry *ge, const fwi_option
                    : (born ? make_tiling(L, pl.ns, STEP_BWD, 0) : make_tiling(L, pl.ns, STEP_BWD));
     if (allow_resident && !pl.snap && !pl.with_offh && !(born && !need_bwd) && op != FWI_OP_GN_HVP)
         pl.rf = choose_resident(L, pl.ns, res_forward_kind(o, op));
-    if (allow_resident && need_bwd && !pl.snap && !pl.ext) pl.rb = choose_resident(L, pl.ns, RES_BWD);
-    // (the workspace does not depend on pinned steps or the receivers' places)
+    if (allow_resident && need_bwd && !pl.snap) pl.rb = choose_resident(L, pl.ns, RES_BWD);
+    // (the workspace does not depend on pinned steps or the receivers' places,
+    // and extended migration holds the state of a plain adjoint pass)
     const size_t xch = (size_t)std::max(pl.rf.xch, pl.rb.xch);
+    if (pl.ext) pl.rb = ResTile{};
     if (pl.rf.ok && (res_pinned(STEP_FWD, L, pl.ns) || (coords && !receivers_fit(L, ge, pl.rf, false)))) pl.rf = ResTile{};
     if (pl.rb.ok && (res_pinned(STEP_BWD, L, pl.ns) || (coords && !receivers_fit(L, ge, pl.rb, true)))) pl.rb = ResTile{};
     const size_t fbytes = (size_t)L.fstride * sizeof(float);
