@@ -171,6 +171,15 @@ typedef struct {
    the traces. opts may be NULL for FWI_OP_FORWARD. */
 fwi_status fwi_workspace_bytes(const fwi_grid *grid, const fwi_geometry *geom,
                                const fwi_options *opts, int op, size_t *bytes);
+/* The workspace with which a call of `op` on nmodels models (more than one:
+   FWI_OP_GRADIENT, as fwi_batch_gradient) takes its fastest path, at least
+   fwi_workspace_bytes() / fwi_batch_workspace_bytes(): small 2-D problems with
+   the offset Hessian keep the levels of their forward pass (at most 4 GiB per
+   model) and sum over them at the end. With less, down to the sizes of those
+   functions, the sums are taken after every level; the results agree to FP32
+   rounding. grids, geoms: HOST arrays [nmodels]. */
+fwi_status fwi_workspace_preferred_bytes(int nmodels, const fwi_grid *grids, const fwi_geometry *geoms,
+                                         const fwi_options *opts, int op, size_t *bytes);
 
 /* Forward modelling of every shot [Sec. 2].
    v     DEVICE [nz][nx] velocity (m/s)

@@ -91,6 +91,7 @@ _SIGS = {
     "fwi_precondition": [P(FwiGrid), c_void_p, c_void_p, c_int, c_int, c_float, c_void_p, c_void_p,
                          c_size_t, c_void_p],
     "fwi_forward_noalloc": [P(FwiGrid), P(FwiGeometry), c_void_p, c_void_p, c_void_p],
+    "fwi_workspace_preferred_bytes": [c_int, P(FwiGrid), P(FwiGeometry), P(FwiOptions), c_int, P(c_size_t)],
     "fwi_batch_workspace_bytes": [c_int, P(FwiGrid), P(FwiGeometry), P(FwiOptions), P(c_size_t)],
     "fwi_batch_gradient": [c_int, P(FwiGrid), P(FwiGeometry), P(FwiOptions), P(c_void_p), P(c_void_p),
                            P(c_void_p), P(c_void_p), c_void_p, P(c_void_p), P(c_void_p), c_void_p,

@@ -101,6 +101,8 @@ struct Plan {
     // the backward pass, and the packets their tiles exchange
     ResTile rf{}, rb{};
     Part xch;
+    Part hist; // resident forward pass with the offset Hessian: its levels, past `total`
+               // (used where the caller's workspace has room, settle_hist)
     size_t total = 0;
 };
 
@@ -224,11 +226,20 @@ double streaming_us(double pts, ResKind kind)
                            : std::min(6.0 + 4.0e-6 * pts, 14.0 + 2.0e-6 * pts);
 }
 
-// The resident time loop where it is expected to be faster
-ResTile choose_resident(const Lay2D &L, int ns, ResKind kind)
+// The levels that a resident forward pass keeps for the offset-Hessian sums
+size_t hist_bytes(const Lay2D &L, int ns, int nt) { return (size_t)(nt - 1) * ns * L.fstride * sizeof(float); }
+constexpr size_t HIST_MAX = size_t(4) << 30;
+
+// The resident time loop where it is expected to be faster; hist > 0: with the
+// offset Hessian, whose sums take about the same time on kept levels (for the
+// writing of which 0.7 us per M points is allowed) as after each streaming step
+// (which adds a launch to each).
+ResTile choose_resident(const Lay2D &L, int ns, ResKind kind, size_t hist = 0)
 {
     const ResTile t = res_plan(L, ns, kind);
-    return t.ok && t.us < streaming_us((double)L.nzp * L.nxp * ns, kind) ? t : ResTile{};
+    const double pts = (double)L.nzp * L.nxp * ns;
+    const double more = hist > 0 ? 0.7e-6 * pts - 4.0 : 0.0;
+    return t.ok && hist <= HIST_MAX && t.us + more < streaming_us(pts, kind) ? t : ResTile{};
 }
 
 ResKind res_forward_kind(const fwi_options *o, int op)
@@ -292,14 +303,16 @@ fwi_status make_plan(const fwi_grid *g, const fwi_geometry *ge, const fwi_option
     // 2 HE + 1 image planes once)
     pl.tb = pl.ext ? make_tiling(L, pl.ns, STEP_BWD, 1, 32)
                    : (born ? make_tiling(L, pl.ns, STEP_BWD, 0) : make_tiling(L, pl.ns, STEP_BWD));
-    if (allow_resident && !pl.snap && !pl.with_offh && !(born && !need_bwd) && op != FWI_OP_GN_HVP)
-        pl.rf = choose_resident(L, pl.ns, res_forward_kind(o, op));
+    if (allow_resident && !pl.snap && !(born && !need_bwd) && op != FWI_OP_GN_HVP)
+        pl.rf = choose_resident(L, pl.ns, res_forward_kind(o, op), pl.with_offh ? hist_bytes(L, pl.ns, pl.nt) : 0);
+    const StepKind fkind = pl.with_offh ? STEP_FWD_OFFH : STEP_FWD;
+    const size_t hist = pl.rf.ok && pl.with_offh ? hist_bytes(L, pl.ns, pl.nt) : 0;
     if (allow_resident && need_bwd && !pl.snap) pl.rb = choose_resident(L, pl.ns, RES_BWD);
     // (the workspace does not depend on pinned steps or the receivers' places,
     // and extended migration holds the state of a plain adjoint pass)
     const size_t xch = (size_t)std::max(pl.rf.xch, pl.rb.xch);
     if (pl.ext) pl.rb = ResTile{};
-    if (pl.rf.ok && (res_pinned(STEP_FWD, L, pl.ns) || (coords && !receivers_fit(L, ge, pl.rf, false)))) pl.rf = ResTile{};
+    if (pl.rf.ok && (res_pinned(fkind, L, pl.ns) || (coords && !receivers_fit(L, ge, pl.rf, false)))) pl.rf = ResTile{};
     if (pl.rb.ok && (res_pinned(STEP_BWD, L, pl.ns) || (coords && !receivers_fit(L, ge, pl.rb, true)))) pl.rb = ResTile{};
     const size_t fbytes = (size_t)L.fstride * sizeof(float);
     const size_t nphys = (size_t)L.nz * L.nx;
@@ -364,8 +377,15 @@ fwi_status make_plan(const fwi_grid *g, const fwi_geometry *ge, const fwi_option
     }
     take(pl.tab, t);
     take(pl.xch, xch);
+    pl.hist = Part{off, hist};
     pl.total = off;
     return FWI_OK;
+}
+
+// a workspace without room for the kept levels: the streaming forward steps
+void settle_hist(Plan &pl, size_t ws_bytes)
+{
+    if (pl.with_offh && ws_bytes < pl.hist.off + pl.hist.bytes) pl.rf = ResTile{};
 }
 
 template <class T> T *at(void *ws, const Part &p) { return reinterpret_cast<T *>(static_cast<char *>(ws) + p.off); }
@@ -655,7 +675,7 @@ ResArgs res_args(const Plan &pl, const fwi_geometry *ge, void *ws, int *status, 
 
 // the whole forward time loop of one model as one resident launch
 fwi_status run_forward_resident(const Plan &pl, const fwi_geometry *ge, void *ws, int *status, float *seis, bool save,
-                                float *acc_i, int illum_utt, cudaStream_t st)
+                                float *acc_i, float *acc_h, int illum_utt, cudaStream_t st)
 {
     cudaError_t e;
     if (acc_i && (e = cudaMemsetAsync(acc_i, 0, pl.acc_i.bytes, st)) != cudaSuccess) return cuda_fail(e, "memset");
@@ -664,10 +684,23 @@ fwi_status run_forward_resident(const Plan &pl, const fwi_geometry *ge, void *ws
     a.save = save;
     a.seis = (seis && pl.nrec > 0) ? seis : nullptr;
     a.acc_illum = acc_i;
+    if (acc_h) {
+        a.hist = at<float>(ws, pl.hist);
+        // (the sums read 12 columns around the model: ghost columns where the
+        // sponge is narrower)
+        if ((e = cudaMemsetAsync(acc_h, 0, pl.acc_h.bytes, st)) != cudaSuccess ||
+            (pl.L.P < HMAX_LIMIT && (e = cudaMemsetAsync(a.hist, 0, pl.hist.bytes, st)) != cudaSuccess))
+            return cuda_fail(e, "memset");
+    }
     const ResKind kind = !acc_i ? RES_FWD : (illum_utt ? RES_FWD_UTT2 : RES_FWD_U2);
     if ((e = launch_resident(a, kind, st)) != cudaSuccess)
         return cuda_fail(e, "resident forward loop");
     t_launch[0]++;
+    if (acc_h) {
+        if ((e = launch_offh_images(pl.L, a.hist, (long long)(pl.nt - 1) * pl.ns, pl.hmax, acc_h, st)) != cudaSuccess)
+            return cuda_fail(e, "offset-Hessian sums");
+        t_launch[0]++;
+    }
     return FWI_OK;
 }
 
@@ -706,7 +739,7 @@ fwi_status run_forward_models(int nm, const Plan *pl, const fwi_geometry *const 
     if (pl[0].rf.ok) { // every model of the call (make_batch)
         for (int k = 0; k < nm; ++k) {
             const fwi_status s = run_forward_resident(pl[k], ge[k], ws[k], at<int>(ws[0], pl[0].scal, 8), seis[k], save,
-                                                      acc_i[k], illum_utt, st);
+                                                      acc_i[k], pl[k].with_offh ? acc_h[k] : nullptr, illum_utt, st);
             if (s != FWI_OK) return s;
         }
         return FWI_OK;
@@ -1805,6 +1838,7 @@ fwi_status make_recv_plan(const fwi_grid *g, const fwi_geometry *ge, const fwi_o
         rp.g2.src = rp.src.data();
     }
     if ((s = make_plan(g, &rp.g2, &rp.o2, FWI_OP_OFFSET_HESSIAN, coords, rp.pl)) != FWI_OK) return s;
+    rp.pl.rf = ResTile{}; // its wavelets follow the plan: no room for kept levels
     rp.wav_off = align_up(rp.pl.total);
     rp.total = rp.wav_off + (size_t)ge->nrec * g->nt * sizeof(float);
     return FWI_OK;
@@ -1824,7 +1858,7 @@ const fwi_options *or_defaults(const fwi_options *o, fwi_options &store)
 }
 
 fwi_status make_batch(int nm, const fwi_grid *grids, const fwi_geometry *geoms, const fwi_options *opts,
-                      bool coords, std::vector<Plan> &pl, std::vector<size_t> &base, size_t &total)
+                      bool coords, std::vector<Plan> &pl, std::vector<size_t> &base, size_t &total, size_t &preferred)
 {
     if (nm < 1 || nm > FWI_BATCH_MAX) return fail(FWI_ERR_INVALID_ARG, "nmodels=%d outside 1..%d", nm, FWI_BATCH_MAX);
     if (!grids || !geoms) return fail(FWI_ERR_INVALID_ARG, "grids or geoms is NULL");
@@ -1842,6 +1876,12 @@ fwi_status make_batch(int nm, const fwi_grid *grids, const fwi_geometry *geoms, 
                         grids[0].nt);
         base[k] = total;
         total = align_up(total + pl[k].total);
+    }
+    // the kept levels of resident forward passes follow the models' slices
+    preferred = total;
+    for (int k = 0; k < nm; ++k) {
+        pl[k].hist.off = preferred - base[k];
+        preferred = align_up(preferred + pl[k].hist.bytes);
     }
     // a launch runs one kernel for all models: the tile variants and chunks
     // of the model with the most work (padded points x shots); the workspace
@@ -2007,6 +2047,7 @@ fwi_status fwi_adjoint_gradient(const fwi_grid *grid, const fwi_geometry *geom, 
     if (!v || !grad || (!d_obs && geom->nrec > 0)) return fail(FWI_ERR_INVALID_ARG, "v, d_obs or grad is NULL");
     if (offh && opts->hmax < 0) return fail(FWI_ERR_INVALID_ARG, "offh requested with hmax < 0");
     if ((s = check_ws(pl, ws, ws_bytes)) != FWI_OK) return s;
+    settle_hist(pl, ws_bytes);
     cudaStream_t st = static_cast<cudaStream_t>(stream);
     GradientIO io{v, d_obs, grad, grad_pre, misfit, illum, offh};
     if ((s = gradient_models(1, &pl, &geom, opts, &ws, &io, st)) != FWI_OK) return s;
@@ -2057,6 +2098,7 @@ fwi_status fwi_offset_hessian_diag(const fwi_grid *grid, const fwi_geometry *geo
     if (s != FWI_OK) return s;
     if (!v || !offh) return fail(FWI_ERR_INVALID_ARG, "v or offh is NULL");
     if ((s = check_ws(pl, ws, ws_bytes)) != FWI_OK) return s;
+    settle_hist(pl, ws_bytes);
     cudaStream_t st = static_cast<cudaStream_t>(stream);
     begin_call(st);
     if ((s = setup(pl, geom, v, ws, st)) != FWI_OK) return s;
@@ -2102,7 +2144,8 @@ fwi_status fwi_precondition(const fwi_grid *grid, const float *grad, const float
     const long long nphys = three ? (long long)grid->nz * grid->ny * grid->nx : (long long)pl.L.nz * pl.L.nx;
     cudaError_t e;
     if ((e = cudaMemsetAsync(at<char>(ws, scal), 0, scal.bytes, st)) != cudaSuccess) return cuda_fail(e, "memset");
-    if ((e = launch_precond_n(nphys, grad, scale, kind, hmax, eps, out, at<unsigned>(ws, scal, 12), st)) != cudaSuccess)
+    if ((e = launch_precond_n(nphys, grad, scale, kind, hmax, eps, out, at<unsigned>(ws, scal, 12), st, true)) !=
+        cudaSuccess)
         return cuda_fail(e, "precondition kernel");
     t_launch[2] += 2;
     prof_record(3, st);
@@ -2643,10 +2686,33 @@ fwi_status fwi_batch_workspace_bytes(int nmodels, const fwi_grid *grids, const f
     if (!bytes) return fail(FWI_ERR_INVALID_ARG, "bytes is NULL");
     std::vector<Plan> pl;
     std::vector<size_t> base;
-    size_t total = 0;
-    fwi_status s = make_batch(nmodels, grids, geoms, opts, false, pl, base, total);
+    size_t total = 0, preferred = 0;
+    fwi_status s = make_batch(nmodels, grids, geoms, opts, false, pl, base, total, preferred);
     if (s != FWI_OK) return s;
     *bytes = total;
+    t_err.clear();
+    return FWI_OK;
+}
+
+fwi_status fwi_workspace_preferred_bytes(int nmodels, const fwi_grid *grids, const fwi_geometry *geoms,
+                                         const fwi_options *opts, int op, size_t *bytes)
+{
+    if (!bytes) return fail(FWI_ERR_INVALID_ARG, "bytes is NULL");
+    const bool two = grids && grids[0].ndim == 2;
+    if (op == FWI_OP_GRADIENT && two && opts && (nmodels > 1 || opts->ckpt == FWI_CKPT_SPONGE)) {
+        std::vector<Plan> pl;
+        std::vector<size_t> base;
+        size_t total = 0;
+        fwi_status s = make_batch(nmodels, grids, geoms, opts, false, pl, base, total, *bytes);
+        if (s == FWI_OK) t_err.clear();
+        return s;
+    }
+    if (nmodels != 1) return fail(FWI_ERR_INVALID_ARG, "nmodels=%d: only 2-D gradients take several models", nmodels);
+    fwi_status s = fwi_workspace_bytes(grids, geoms, opts, op, bytes);
+    if (s != FWI_OK || op != FWI_OP_OFFSET_HESSIAN || !two) return s;
+    Plan pl;
+    if ((s = make_plan(grids, geoms, opts, op, false, pl)) != FWI_OK) return s;
+    *bytes = pl.hist.off + pl.hist.bytes;
     t_err.clear();
     return FWI_OK;
 }
@@ -2668,8 +2734,8 @@ fwi_status batch_prepare(int nmodels, const fwi_grid *grids, const fwi_geometry 
                          size_t ws_bytes, BatchCall &bc)
 {
     std::vector<size_t> base;
-    size_t total = 0;
-    fwi_status s = make_batch(nmodels, grids, geoms, opts, true, bc.pl, base, total);
+    size_t total = 0, preferred = 0;
+    fwi_status s = make_batch(nmodels, grids, geoms, opts, true, bc.pl, base, total, preferred);
     if (s != FWI_OK) return s;
     if (!v || !grad || !d_obs) return fail(FWI_ERR_INVALID_ARG, "v, d_obs or grad is NULL");
     std::vector<GradientIO> &io = bc.io;
@@ -2685,6 +2751,9 @@ fwi_status batch_prepare(int nmodels, const fwi_grid *grids, const fwi_geometry 
         wk[k] = static_cast<char *>(ws) + base[k];
     }
     if ((s = check_ws_bytes(ws, ws_bytes, total)) != FWI_OK) return s;
+    if (ws_bytes < preferred)
+        for (Plan &p : bc.pl)
+            if (p.with_offh) p.rf = ResTile{};
     bc.gp.assign(nmodels, nullptr);
     for (int k = 0; k < nmodels; ++k) bc.gp[k] = &geoms[k];
     return FWI_OK;

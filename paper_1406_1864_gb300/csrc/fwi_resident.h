@@ -47,6 +47,7 @@ struct ResArgs {
     float *seis;           // [ns][nt][nrec] or null
     float *acc_illum;      // [nz][nx] or null
     int save;              // the final two levels are written to u
+    float *hist;           // levels 1 .. nt - 1 of every shot ([nt - 1][ns] fields) or null
     // backward
     const float *adj;      // [nt][nent], receiver-table order, or null
     int nent;
@@ -61,6 +62,9 @@ ResTile res_plan(const Lay2D &L, int ns, ResKind kind);
 void res_pin(StepKind kind, const Lay2D &L, int ns, bool pinned);
 bool res_pinned(StepKind kind, const Lay2D &L, int ns);
 void res_pin_clear();
+// acc[h][x] += sum over n images (field layout, fstride apart) of u(x + h) u(x - h),
+// h = 0 .. hmax, at the physical points
+cudaError_t launch_offh_images(const Lay2D &L, const float *u, long long n, int hmax, float *acc, cudaStream_t st);
 cudaError_t launch_resident(const ResArgs &a, ResKind kind, cudaStream_t st);
 
 } // namespace fwi

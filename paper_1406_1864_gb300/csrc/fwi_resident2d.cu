@@ -653,15 +653,64 @@ __device__ __forceinline__ void fwd_rows(const float *f, float *g, const float4 
     }
 }
 
+// Sums of u^2 and of the imaging factor are taken in registers over RES_SUM
+// levels of the shots in flight and then added to memory: sums over a whole
+// pass (2000 terms at 2 shots and nt 1000) rounded to 1.5e-6, streaming 1e-6.
+constexpr int RES_SUM = 32;
+
+template <int R>
+__device__ __forceinline__ void flush_illum(const ResArgs &a, const Own<R> &o, float2 (&acc)[R][2])
+{
+    const Lay2D &L = a.L;
+#pragma unroll
+    for (int r = 0; r < R; ++r) {
+        const int iz = o.i0 + r - L.P, ix0 = o.j0 - L.P;
+        if (o.on && iz >= 0 && iz < L.nz) {
+            float *p = a.acc_illum + (long long)iz * L.nx + ix0;
+            if (((L.P | L.nx) & 3) == 0) {
+                if (ix0 >= 0 && ix0 + 3 < L.nx) red_add4(p, acc[r][0].x, acc[r][0].y, acc[r][1].x, acc[r][1].y);
+            } else {
+                if (ix0 >= 0 && ix0 < L.nx) atomicAdd(p, acc[r][0].x);
+                if (ix0 + 1 >= 0 && ix0 + 1 < L.nx) atomicAdd(p + 1, acc[r][0].y);
+                if (ix0 + 2 >= 0 && ix0 + 2 < L.nx) atomicAdd(p + 2, acc[r][1].x);
+                if (ix0 + 3 >= 0 && ix0 + 3 < L.nx) atomicAdd(p + 3, acc[r][1].y);
+            }
+        }
+        acc[r][0] = acc[r][1] = make_float2(0.f, 0.f);
+    }
+}
+
+template <int R>
+__device__ __forceinline__ void flush_grad(const ResArgs &a, const Own<R> &o, float2 (&acc)[R][2])
+{
+    const Lay2D &L = a.L;
+#pragma unroll
+    for (int r = 0; r < R; ++r) {
+        if (o.in >> r & 1) {
+            float *p = a.acc_grad + (long long)(o.i0 + r) * L.nxp + o.j0;
+            if ((L.nxp & 3) == 0) {
+                red_add4(p, acc[r][0].x, acc[r][0].y, acc[r][1].x, acc[r][1].y);
+            } else {
+                atomicAdd(p, acc[r][0].x);
+                if (o.j0 + 1 < L.nxp) atomicAdd(p + 1, acc[r][0].y);
+                if (o.j0 + 2 < L.nxp) atomicAdd(p + 2, acc[r][1].x);
+                if (o.j0 + 3 < L.nxp) atomicAdd(p + 3, acc[r][1].y);
+            }
+        }
+        acc[r][0] = acc[r][1] = make_float2(0.f, 0.f);
+    }
+}
+
 // The compute warps' time loop over one round of shots: shots g, g + G, ... of
 // the warp's group g.
 template <int R, int G, int MODE, int ACC>
 __device__ __forceinline__ bool fwd_loop(const ResArgs &a, const Own<R> &o, float *sm, const float4 (&ca)[R], const float *kb,
-                                         float2 (&acc)[R][2], ResShared &sh, int group, int nsh, unsigned srcs, uint32_t pf)
+                                         float2 (&acc)[R][2], ResShared &sh, int group, int shot0, int nsh, unsigned srcs, uint32_t pf)
 {
     const int nt = a.nt, fs = a.t.fs, lane = threadIdx.x & 31;
     for (int n = 0; n < nt; ++n) {
         const uint32_t par = (pf + n) & 1u;
+        if (ACC && n > 0 && n % RES_SUM == 0) flush_illum<R>(a, o, acc);
         for (int s = group; s < nsh; s += G) {
             if (!res_wait(smem_u32(&sh.bars.full[s]), par, &sh.abort)) return false;
             const float *f = sm + (2 * s + (n & 1)) * fs + o.so;
@@ -705,6 +754,15 @@ __device__ __forceinline__ bool fwd_loop(const ResArgs &a, const Own<R> &o, floa
             }
             __syncwarp();
             if (lane == 0) mbar_arrive(smem_u32(&sh.bars.done[s]));
+            // the level for the offset-Hessian sums, after the others may go on
+            // (this thread's own points: only its next step on this buffer, two
+            // levels on, overwrites them)
+            if (a.hist != nullptr && o.on) {
+                float *hp = a.hist + ((long long)n * a.ns + shot0 + s) * a.L.fstride + fidx(a.L, o.i0, o.j0);
+#pragma unroll
+                for (int r = 0; r < R; ++r)
+                    if (o.in >> r & 1) *reinterpret_cast<float4 *>(hp + r * a.L.pitch) = lds4(g + r * RES_P);
+            }
         }
     }
     return true;
@@ -770,26 +828,9 @@ __global__ void __launch_bounds__(32 * (NW + RES_SVC), 1) k_fwd_resident(const _
                     srcs |= 1u << s;
             const uint32_t pf = (uint32_t)(round * nt);
             const bool ok = __any_sync(0xffffffffu, o.bmask != 0)
-                ? fwd_loop<R, G, 1, ACC>(a, o, sm, ca, kbs + o.ko, acc, sh, group, nsh, srcs, pf)
-                : fwd_loop<R, G, 0, ACC>(a, o, sm, ca, kbs + o.ko, acc, sh, group, nsh, srcs, pf);
-            if (ACC && ok && o.on) {
-                // the round's sums into the physical grid
-#pragma unroll
-                for (int r = 0; r < R; ++r) {
-                    const int iz = o.i0 + r - L.P, ix0 = o.j0 - L.P;
-                    if (iz < 0 || iz >= L.nz) continue;
-                    if (((L.P | L.nx) & 3) == 0) {
-                        if (ix0 >= 0 && ix0 + 3 < L.nx)
-                            red_add4(a.acc_illum + (long long)iz * L.nx + ix0, acc[r][0].x, acc[r][0].y, acc[r][1].x,
-                                     acc[r][1].y);
-                    } else {
-                        const float v[4] = {acc[r][0].x, acc[r][0].y, acc[r][1].x, acc[r][1].y};
-#pragma unroll
-                        for (int p = 0; p < 4; ++p)
-                            if (ix0 + p >= 0 && ix0 + p < L.nx) atomicAdd(a.acc_illum + (long long)iz * L.nx + ix0 + p, v[p]);
-                    }
-                }
-            }
+                ? fwd_loop<R, G, 1, ACC>(a, o, sm, ca, kbs + o.ko, acc, sh, group, first + base, nsh, srcs, pf)
+                : fwd_loop<R, G, 0, ACC>(a, o, sm, ca, kbs + o.ko, acc, sh, group, first + base, nsh, srcs, pf);
+            if (ACC && ok) flush_illum<R>(a, o, acc);
             // the last two levels: checked, and kept for an adjoint pass
             if (ok && o.on) {
                 bool fin = true;
@@ -957,6 +998,7 @@ __device__ __forceinline__ bool bwd_loop(const ResArgs &a, const Own<R> &o, floa
     const int nt = a.nt, fs = a.t.fs, lane = threadIdx.x & 31;
     for (int m = nt - 1; m >= 1; --m) {
         const int step = nt - 1 - m, pc = (m - 1) & 1, pn = m & 1, par = step & 1;
+        if (step > 0 && step % RES_SUM == 0) flush_grad<R>(a, o, acc);
         for (int s = group; s < nsh; s += G) {
             if (!res_wait(smem_u32(&sh.bars.full[s]), (pf + step) & 1u, &sh.abort)) return false;
             if (o.on) {
@@ -1068,21 +1110,7 @@ __global__ void __launch_bounds__(32 * (NW + RES_SVC), 1) k_bwd_resident(const _
                 ok = bwd_loop<R, G, 1>(a, o, sm, ca, kbs + o.ko, acc, sh, inj, group, nsh, srcs, pf);
             else
                 ok = bwd_loop<R, G, 0>(a, o, sm, ca, kbs + o.ko, acc, sh, inj, group, nsh, srcs, pf);
-            if (ok && o.on) {
-#pragma unroll
-                for (int r = 0; r < R; ++r) {
-                    if (!(o.in >> r & 1)) continue;
-                    float *g = a.acc_grad + (long long)(o.i0 + r) * L.nxp + o.j0;
-                    if ((L.nxp & 3) == 0) {
-                        red_add4(g, acc[r][0].x, acc[r][0].y, acc[r][1].x, acc[r][1].y);
-                    } else {
-                        const float v[4] = {acc[r][0].x, acc[r][0].y, acc[r][1].x, acc[r][1].y};
-#pragma unroll
-                        for (int p = 0; p < 4; ++p)
-                            if (o.j0 + p < L.nxp) atomicAdd(g + p, v[p]);
-                    }
-                }
-            }
+            if (ok) flush_grad<R>(a, o, acc);
             if (ok && o.on) {
                 bool fin = true;
                 for (int s = group; s < nsh; s += G)
@@ -1107,6 +1135,100 @@ __global__ void __launch_bounds__(32 * (NW + RES_SVC), 1) k_bwd_resident(const _
             if (threadIdx.x == 0) atomicOr(a.status, ST_TIMEOUT);
             return;
         }
+    }
+}
+
+// ----------------------------------------- offset Hessian of kept levels
+// The offset-Hessian sums of a resident forward pass: its registers hold no 11
+// or 13 sums per point, so the pass keeps its levels (small problems only) and
+// this kernel sums the products of all of them at once: a CTA takes a 64 x 8 tile
+// of the physical points and a run of images, whose rows with 12 columns on each
+// side go through two shared-memory stages of OI images; each thread holds the
+// sums of its 4 points over the run. Bound by shared memory: 7 16-byte reads per
+// 4 points and image.
+constexpr int OI = 4, OI_W = TX + 2 * HMAX_LIMIT;
+
+template <int NHC>
+__global__ void __launch_bounds__(TPB, 4) k_offh_images(const float *__restrict__ u, const __grid_constant__ Lay2D L,
+                                                        long long n, int run, int hmax, float *acc_offh)
+{
+    constexpr int WL = HMAX_LIMIT, NW4 = (2 * WL + 4) / 4;
+    __shared__ __align__(16) float sm[2][OI][8 * OI_W];
+    const int ntx = (L.nx + TX - 1) / TX, ntz = (L.nz + 7) / 8;
+    const int c = blockIdx.x / (ntx * ntz), tile = blockIdx.x - c * (ntx * ntz), bz = tile / ntx, bx = tile - bz * ntx;
+    const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4, iz0 = 8 * bz, ixb = TX * bx;
+    const long long k0 = (long long)c * run, k1 = min(n, k0 + run);
+    const bool al = (L.P & 3) == 0;
+    // images k .. k + OI - 1 into stage b; cells below the model or past the
+    // last column's offsets belong to points that are not stored
+    auto stage = [&](long long k, int b) {
+#pragma unroll 1
+        for (int q = 0; q < OI && k + q < k1; ++q) {
+            const float *src = u + (k + q) * L.fstride;
+            float *dst = sm[b][q];
+            if (al) {
+                for (int e = threadIdx.x; e < 8 * (OI_W / 4); e += TPB) {
+                    const int r = e / (OI_W / 4), c4 = 4 * (e - r * (OI_W / 4)), col = ixb - WL + c4;
+                    if (iz0 + r < L.nz && col < L.nx + WL) copy16(dst + r * OI_W + c4, src + fidx(L, iz0 + r + L.P, col + L.P));
+                }
+            } else {
+                for (int e = threadIdx.x; e < 8 * OI_W; e += TPB) {
+                    const int r = e / OI_W, cc = e - r * OI_W, col = ixb - WL + cc;
+                    if (iz0 + r < L.nz && col < L.nx + WL) copy4(dst + r * OI_W + cc, src + fidx(L, iz0 + r + L.P, col + L.P));
+                }
+            }
+        }
+        copies_commit();
+    };
+    float2 acc[NHC][2];
+#pragma unroll
+    for (int h = 0; h < NHC; ++h) acc[h][0] = acc[h][1] = make_float2(0.f, 0.f);
+    stage(k0, 0);
+    int b = 0;
+    for (long long k = k0; k < k1; k += OI, b ^= 1) {
+        if (k + OI < k1) stage(k + OI, b ^ 1);
+        else copies_commit();
+        copies_wait_but(1);
+        __syncthreads();
+        const int nq = (int)min((long long)OI, k1 - k);
+#pragma unroll 1
+        for (int q = 0; q < nq; ++q) {
+            const float *row = &sm[b][q][ty * OI_W + 4 * tx];
+            float w[4 * NW4];
+#pragma unroll
+            for (int e = 0; e < NW4; ++e) {
+                const float4 t = lds4(row + 4 * e);
+                w[4 * e] = t.x; w[4 * e + 1] = t.y; w[4 * e + 2] = t.z; w[4 * e + 3] = t.w;
+            }
+            // even h: points (0, 1), (2, 3) on lane pairs; odd h: (1, 2) paired, 0 and 3 scalar
+#pragma unroll
+            for (int h = 0; h < NHC; ++h) {
+                if ((h & 1) == 0) {
+#pragma unroll
+                    for (int y = 0; y < 2; ++y)
+                        acc[h][y] = fma2(f2(w[WL + 2 * y + h], w[WL + 2 * y + 1 + h]),
+                                         f2(w[WL + 2 * y - h], w[WL + 2 * y + 1 - h]), acc[h][y]);
+                } else {
+                    acc[h][0] = fma2(f2(w[WL + 1 + h], w[WL + 2 + h]), f2(w[WL + 1 - h], w[WL + 2 - h]), acc[h][0]);
+                    acc[h][1].x = fmaf(w[WL + h], w[WL - h], acc[h][1].x);
+                    acc[h][1].y = fmaf(w[WL + 3 + h], w[WL + 3 - h], acc[h][1].y);
+                }
+            }
+        }
+        __syncthreads(); // stage b is free
+    }
+    copies_wait();
+    const int iz = iz0 + ty, ix0 = ixb + 4 * tx;
+    if (iz >= L.nz || ix0 >= L.nx) return;
+    const long long nphys = (long long)L.nz * L.nx, at = (long long)iz * L.nx + ix0;
+#pragma unroll
+    for (int h = 0; h < NHC; ++h) {
+        if (h > hmax) continue;
+        const float v[4] = {(h & 1) ? acc[h][1].x : acc[h][0].x, (h & 1) ? acc[h][0].x : acc[h][0].y,
+                            (h & 1) ? acc[h][0].y : acc[h][1].x, acc[h][1].y};
+#pragma unroll
+        for (int p = 0; p < 4; ++p)
+            if (ix0 + p < L.nx) atomicAdd(acc_offh + h * nphys + at + p, v[p]);
     }
 }
 
@@ -1248,6 +1370,26 @@ void res_pin_clear()
 {
     std::lock_guard<std::mutex> lock(g_pin_mu);
     g_pinned.clear();
+}
+
+cudaError_t launch_offh_images(const Lay2D &L, const float *u, long long n, int hmax, float *acc, cudaStream_t st)
+{
+    if (n <= 0) return cudaSuccess;
+    res_prepare();
+    // runs of images such that the tiles fill the SMs' 4 CTAs about twice, of at
+    // least 32 images (each run adds its sums to memory once) and at most 256
+    // (FP32 sums of more images lose digits that the sum over runs keeps)
+    const long long tiles = (long long)((L.nz + 7) / 8) * ((L.nx + TX - 1) / TX);
+    const long long runs = std::max<long long>(1, 8LL * g_res_sms / tiles);
+    const int run = (int)std::max<long long>(32, std::min<long long>(256, (n + runs - 1) / runs));
+    const unsigned grid = (unsigned)(tiles * ((n + run - 1) / run));
+    if (hmax <= 3)
+        k_offh_images<4><<<grid, TPB, 0, st>>>(u, L, n, run, hmax, acc);
+    else if (hmax <= 10)
+        k_offh_images<11><<<grid, TPB, 0, st>>>(u, L, n, run, hmax, acc);
+    else
+        k_offh_images<13><<<grid, TPB, 0, st>>>(u, L, n, run, hmax, acc);
+    return cudaGetLastError();
 }
 
 cudaError_t launch_resident(const ResArgs &a, ResKind kind, cudaStream_t st)

@@ -133,6 +133,19 @@ def workspace_bytes(grid: Grid, geom: Geometry, opts: Options | None, op: str) -
     return int(n.value)
 
 
+def preferred_workspace_bytes(grids, geoms, opts: Options, op: str) -> int:
+    """fwi_workspace_preferred_bytes: the size with which the call takes its
+    fastest path (the functions below ask for it where they allocate)."""
+    n = len(grids)
+    g = (L.FwiGrid * n)(*[x.c() for x in grids])
+    ge = (L.FwiGeometry * n)(*[x.c() for x in geoms])
+    oc = opts.c()
+    nb = ctypes.c_size_t(0)
+    L.check(L.load().fwi_workspace_preferred_bytes(n, g, ge, ctypes.byref(oc), OPS[op], ctypes.byref(nb)),
+            "fwi_workspace_preferred_bytes")
+    return int(nb.value)
+
+
 class Workspace:
     """A reusable device workspace (grows on demand)."""
 
@@ -206,7 +219,7 @@ def adjoint_gradient(grid: Grid, geom: Geometry, v: torch.Tensor, d_obs: torch.T
     if want_offh:
         res["offh"] = o.get("offh", torch.empty((opts.hmax + 1,) + grid.shape, dtype=torch.float32,
                                                 device=dev))
-    buf, nb = _ws(ws, workspace_bytes(grid, geom, opts, "gradient"))
+    buf, nb = _ws(ws, preferred_workspace_bytes([grid], [geom], opts, "gradient"))
     g, ge, oc = grid.c(), geom.c(), opts.c()
     L.check(L.load().fwi_adjoint_gradient(
         ctypes.byref(g), ctypes.byref(ge), ctypes.byref(oc), _ptr(v), _ptr(d_obs), _ptr(res["grad"]),
@@ -267,7 +280,7 @@ def batch_gradient(grids, geoms, vs, d_obs, opts: Options | None = None, *, want
     Returns one dict per model, as adjoint_gradient."""
     opts = opts or Options()
     res, c = _batch_args(grids, geoms, vs, d_obs, opts, want_pre, want_illum, want_offh)
-    buf, nb = _ws(ws, batch_workspace_bytes(grids, geoms, opts))
+    buf, nb = _ws(ws, preferred_workspace_bytes(grids, geoms, opts, "gradient"))
     L.check(L.load().fwi_batch_gradient(len(grids), c["g"], c["ge"], ctypes.byref(c["o"]), c["v"], c["d"],
                                         c["grad"], c["pre"], _ptr(c["misfit"]), c["ill"], c["off"], _ptr(buf),
                                         nb, _stream(stream)), "fwi_batch_gradient")
@@ -287,7 +300,7 @@ class GradientGraph:
         self.inputs = (list(vs), list(d_obs))
         self.results, c = _batch_args(grids, geoms, vs, d_obs, opts, want_pre, want_illum, want_offh)
         self._c = c  # keep the ctypes arrays alive with the graph
-        self.buf, nb = _ws(ws, batch_workspace_bytes(grids, geoms, opts))
+        self.buf, nb = _ws(ws, preferred_workspace_bytes(grids, geoms, opts, "gradient"))
         self.stream = torch.cuda.Stream(device=vs[0].device)
         self.stream.wait_stream(torch.cuda.current_stream())
         h = ctypes.c_void_p(0)
@@ -434,7 +447,7 @@ def offset_hessian_diag(grid: Grid, geom: Geometry, v: torch.Tensor, opts: Optio
     offset-Hessian diagonal, offsets along x."""
     _dev(v, "v", grid.shape)
     out = torch.empty((opts.hmax + 1,) + grid.shape, dtype=torch.float32, device=v.device)
-    buf, nb = _ws(ws, workspace_bytes(grid, geom, opts, "offset_hessian"))
+    buf, nb = _ws(ws, preferred_workspace_bytes([grid], [geom], opts, "offset_hessian"))
     g, ge, oc = grid.c(), geom.c(), opts.c()
     L.check(L.load().fwi_offset_hessian_diag(ctypes.byref(g), ctypes.byref(ge), ctypes.byref(oc),
                                              _ptr(v), _ptr(out), _ptr(buf), nb, _stream(stream)),

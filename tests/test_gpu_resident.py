@@ -118,3 +118,29 @@ def test_crowded_tiles_take_the_streaming_adjoint(torch_cuda):
     opts = fwi.Options()
     a, b = both(fwi, grid, geom, opts, lambda: fwi.adjoint_gradient(grid, geom, v, d, opts))
     assert rel(a["grad"], b["grad"]) <= 1e-6
+
+
+@pytest.mark.parametrize("hmax", [0, 3, 10, 12])
+@pytest.mark.parametrize("nz,nx,ns,nt,P", [(37, 83, 3, 60, 7), (50, 130, 5, 40, 20), (8, 65, 1, 30, 1), (23, 64, 9, 70, 16)])
+def test_offset_hessian_of_kept_levels(torch_cuda, nz, nx, ns, nt, P, hmax):
+    """The offset-Hessian sums over the levels a resident pass keeps against
+    those after each streaming step: widths around the 64-column tile, sponges
+    narrower and wider than the 12 columns the sums read on each side, each
+    compiled offset count, a last run of images that is not full. Both add the
+    same FP32 products (at most 630 per point) in another order: 1e-5 is three
+    times their random-walk rounding, 2^-24 sqrt(630) per side, in L2."""
+    from paper_1406_1864_gb300 import fwi
+    torch = torch_cuda
+    grid, geom, v, d = problem(torch, nz, nx, ns, nt, P)
+    opts = fwi.Options(hmax=hmax, precond="offset")
+    a, b = both(fwi, grid, geom, opts, lambda: (fwi.adjoint_gradient(grid, geom, v, d, opts),
+                                                fwi.offset_hessian_diag(grid, geom, v, opts)))
+    for k in ("offh", "illum", "grad"):
+        assert rel(a[0][k], b[0][k]) <= 1e-5, k
+    assert rel(a[1], b[1]) <= 1e-5
+    assert rel(a[0]["offh"][0], a[0]["illum"]) <= 1e-5
+    # a workspace without room for the levels: the sums after each level
+    small = torch.empty(fwi.workspace_bytes(grid, geom, opts, "gradient"), dtype=torch.uint8, device="cuda")
+    assert small.numel() < fwi.preferred_workspace_bytes([grid], [geom], opts, "gradient")
+    c = fwi.adjoint_gradient(grid, geom, v, d, opts, ws=small)
+    assert rel(c["offh"], b[0]["offh"]) <= 1e-5 and rel(c["grad"], b[0]["grad"]) <= 1e-5
