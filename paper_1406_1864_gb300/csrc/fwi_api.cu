@@ -260,6 +260,7 @@ fwi_status make_plan(const fwi_grid *g, const fwi_geometry *ge, const fwi_option
     if ((st = check_opts(o, op)) != FWI_OK) return st;
     pl.L = make_layout(g);
     pl.rf = pl.rb = ResTile{};
+    pl.hist = Part{};
     pl.op = op;
     pl.nt = g->nt;
     const Lay2D &L = pl.L;
@@ -303,7 +304,8 @@ fwi_status make_plan(const fwi_grid *g, const fwi_geometry *ge, const fwi_option
     // 2 HE + 1 image planes once)
     pl.tb = pl.ext ? make_tiling(L, pl.ns, STEP_BWD, 1, 32)
                    : (born ? make_tiling(L, pl.ns, STEP_BWD, 0) : make_tiling(L, pl.ns, STEP_BWD));
-    if (allow_resident && !pl.snap && !(born && !need_bwd) && op != FWI_OP_GN_HVP)
+    // (16-bit snapshots are scaled by the maxima of a whole field: streaming)
+    if (allow_resident && (!pl.snap || o->snap_prec == FWI_SNAP_F32) && !(born && !need_bwd) && op != FWI_OP_GN_HVP)
         pl.rf = choose_resident(L, pl.ns, res_forward_kind(o, op), pl.with_offh ? hist_bytes(L, pl.ns, pl.nt) : 0);
     const StepKind fkind = pl.with_offh ? STEP_FWD_OFFH : STEP_FWD;
     const size_t hist = pl.rf.ok && pl.with_offh ? hist_bytes(L, pl.ns, pl.nt) : 0;
@@ -311,6 +313,7 @@ fwi_status make_plan(const fwi_grid *g, const fwi_geometry *ge, const fwi_option
     // (the workspace does not depend on pinned steps or the receivers' places,
     // and extended migration holds the state of a plain adjoint pass)
     const size_t xch = (size_t)std::max(pl.rf.xch, pl.rb.xch);
+    const size_t acc_groups = pl.rf.ok ? pl.rf.accs : 1;
     if (pl.ext) pl.rb = ResTile{};
     if (pl.rf.ok && (res_pinned(fkind, L, pl.ns) || (coords && !receivers_fit(L, ge, pl.rf, false)))) pl.rf = ResTile{};
     if (pl.rb.ok && (res_pinned(STEP_BWD, L, pl.ns) || (coords && !receivers_fit(L, ge, pl.rb, true)))) pl.rb = ResTile{};
@@ -355,7 +358,7 @@ fwi_status make_plan(const fwi_grid *g, const fwi_geometry *ge, const fwi_option
     if (op == FWI_OP_GRADIENT || op == FWI_OP_GN_HVP || op == FWI_OP_MISFIT) take(pl.syn, (size_t)pl.ns * pl.nt * pl.nrec * sizeof(float));
     if (pl.need_bwd) take(pl.adj_t, (size_t)pl.ns * pl.nt * pl.nrec * sizeof(float));
     if (op == FWI_OP_GRADIENT || op == FWI_OP_ILLUMINATION)
-        take(pl.acc_i, nphys * sizeof(float));
+        take(pl.acc_i, nphys * sizeof(float) * acc_groups);
     if (pl.with_offh) take(pl.acc_h, (size_t)(pl.hmax + 1) * nphys * sizeof(float));
     // tables: src offsets, receiver CSR of the forward and backward tilings
     size_t t = 0;
@@ -680,8 +683,15 @@ fwi_status run_forward_resident(const Plan &pl, const fwi_geometry *ge, void *ws
     cudaError_t e;
     if (acc_i && (e = cudaMemsetAsync(acc_i, 0, pl.acc_i.bytes, st)) != cudaSuccess) return cuda_fail(e, "memset");
     ResArgs a = res_args(pl, ge, ws, status, 0);
-    a.band = save ? at<float>(ws, pl.band) : nullptr;
-    a.save = save;
+    a.band = save && !pl.snap ? at<float>(ws, pl.band) : nullptr;
+    a.save = save && !pl.snap;
+    if (save && pl.snap) {
+        // (a snapshot is restored with its ghost frame)
+        if ((e = cudaMemsetAsync(at<char>(ws, pl.snaps), 0, pl.snaps.bytes, st)) != cudaSuccess)
+            return cuda_fail(e, "memset");
+        a.snaps = at<float>(ws, pl.snaps);
+        a.snap_k = pl.K;
+    }
     a.seis = (seis && pl.nrec > 0) ? seis : nullptr;
     a.acc_illum = acc_i;
     if (acc_h) {
@@ -1098,7 +1108,7 @@ fwi_status gradient_models(int nm, const Plan *pl, const fwi_geometry *const *ge
         const float iscale = opts->illum_mode == FWI_ILLUM_U2 ? p.L.dt : 1.0f / (p.L.dt * p.L.dt * p.L.dt);
         float *ill_out = o.illum ? o.illum : acc_i[k]; // in place into group 0 when not requested
         const float *v6 = opts->hess_v6 ? o.v : nullptr;
-        if ((e = launch_finish_accum(p.L, acc_i[k], 1, 1, iscale, ill_out, st, v6)) != cudaSuccess)
+        if ((e = launch_finish_accum(p.L, acc_i[k], p.rf.ok ? p.rf.accs : 1, 1, iscale, ill_out, st, v6)) != cudaSuccess)
             return cuda_fail(e, "illumination output");
         t_launch[2]++;
         float *off_out = nullptr;
@@ -2077,7 +2087,7 @@ fwi_status fwi_illumination(const fwi_grid *grid, const fwi_geometry *geom, cons
     prof_record(2, st);
     const float iscale = opts->illum_mode == FWI_ILLUM_U2 ? pl.L.dt : 1.0f / (pl.L.dt * pl.L.dt * pl.L.dt);
     cudaError_t e;
-    if ((e = launch_finish_accum(pl.L, acc_i, 1, 1, iscale, illum, st, opts->hess_v6 ? v : nullptr)) != cudaSuccess)
+    if ((e = launch_finish_accum(pl.L, acc_i, pl.rf.ok ? pl.rf.accs : 1, 1, iscale, illum, st, opts->hess_v6 ? v : nullptr)) != cudaSuccess)
         return cuda_fail(e, "illumination output");
     t_launch[2]++;
     prof_record(3, st);
@@ -2268,6 +2278,11 @@ fwi_status fwi_plessix_mulder_hessian(const fwi_grid *grid, const fwi_geometry *
         g.rec = geom->rec + s0 * nrec3;
         g.wavelet = geom->wavelet + (size_t)s0 * grid->nt;
         if ((s = make_plan(grid, &g, opts, FWI_OP_ILLUMINATION, true, pr)) != FWI_OK) return s;
+        // (a resident pass over few shots may be laid out over more sets and tiles
+        // than that of all shots: streaming steps where it does not fit their plan)
+        if (align_up(pr.total) > align_up(all.total) &&
+            (s = make_plan(grid, &g, opts, FWI_OP_ILLUMINATION, true, pr, false)) != FWI_OK)
+            return s;
         if (run == 0) {
             if ((s = setup(pr, &g, v, ws, st)) != FWI_OK) return s;
         } else {
@@ -2283,7 +2298,7 @@ fwi_status fwi_plessix_mulder_hessian(const fwi_grid *grid, const fwi_geometry *
         float *acc_i = at<float>(ws, pr.acc_i);
         if ((e = cudaMemsetAsync(acc_i, 0, pr.acc_i.bytes, st)) != cudaSuccess) return cuda_fail(e, "memset");
         if ((s = run_forward(pr, &g, ws, nullptr, false, acc_i, nullptr, mode, st)) != FWI_OK) return s;
-        if ((e = launch_finish_accum(pr.L, acc_i, 1, 1, iscale, tmp, st, opts->hess_v6 ? v : nullptr)) !=
+        if ((e = launch_finish_accum(pr.L, acc_i, pr.rf.ok ? pr.rf.accs : 1, 1, iscale, tmp, st, opts->hess_v6 ? v : nullptr)) !=
             cudaSuccess)
             return cuda_fail(e, "illumination output");
         int xmin, xmax;
@@ -2699,7 +2714,7 @@ fwi_status fwi_workspace_preferred_bytes(int nmodels, const fwi_grid *grids, con
 {
     if (!bytes) return fail(FWI_ERR_INVALID_ARG, "bytes is NULL");
     const bool two = grids && grids[0].ndim == 2;
-    if (op == FWI_OP_GRADIENT && two && opts && (nmodels > 1 || opts->ckpt == FWI_CKPT_SPONGE)) {
+    if (op == FWI_OP_GRADIENT && two && opts) {
         std::vector<Plan> pl;
         std::vector<size_t> base;
         size_t total = 0;

@@ -21,6 +21,8 @@ struct ResTile {
     int w4, th, g;     // float4 columns, rows, row groups of a tile
     int ntx, ntz;      // tiles of one shot
     int sets, s;       // CTA groups; shots in flight per CTA
+    int accs;          // illumination sums held apart: one per set and group of warps,
+                       // so that each is added to in a fixed order
     int per;           // shots of one set over the whole pass
     int fs;            // floats of one field tile with its halo
     int ne;            // float4s of a tile's edge strips
@@ -45,8 +47,10 @@ struct ResArgs {
     float *band;           // [ns][nt][nbandp]
     // forward
     float *seis;           // [ns][nt][nrec] or null
-    float *acc_illum;      // [nz][nx] or null
+    float *acc_illum;      // [accs][nz][nx] or null
     int save;              // the final two levels are written to u
+    float *snaps;          // F32 snapshots (u^n, u^{n-1}) at n = 0, snap_k, ..., [.][2][ns] fields, or null
+    int snap_k;
     float *hist;           // levels 1 .. nt - 1 of every shot ([nt - 1][ns] fields) or null
     // backward
     const float *adj;      // [nt][nent], receiver-table order, or null

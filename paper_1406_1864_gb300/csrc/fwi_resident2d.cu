@@ -37,7 +37,7 @@
 // Arithmetic. The updates are the streaming steps' own (lap4, lane pairs), so
 // wavefields, checkpoints and traces are bitwise the same; only the order in
 // which shots and levels are summed differs (illumination and imaging sums
-// stay in registers over the S shots and all levels). Cells of a tile outside
+// stay in registers over the S shots and up to RES_SUM levels). Cells of a tile outside
 // the padded grid have c2 = 0 and stay zero.
 //
 // Bound and measured. Per 128 points of a row the forward update is 112 cycles of
@@ -659,15 +659,15 @@ __device__ __forceinline__ void fwd_rows(const float *f, float *g, const float4 
 constexpr int RES_SUM = 32;
 
 template <int R>
-__device__ __forceinline__ void flush_illum(const ResArgs &a, const Own<R> &o, float2 (&acc)[R][2])
+__device__ __forceinline__ void flush_illum(const ResArgs &a, const Own<R> &o, float2 (&acc)[R][2], int group)
 {
     const Lay2D &L = a.L;
 #pragma unroll
     for (int r = 0; r < R; ++r) {
         const int iz = o.i0 + r - L.P, ix0 = o.j0 - L.P;
         if (o.on && iz >= 0 && iz < L.nz) {
-            float *p = a.acc_illum + (long long)iz * L.nx + ix0;
-            if (((L.P | L.nx) & 3) == 0) {
+            float *p = a.acc_illum + ((long long)group * L.nz + iz) * L.nx + ix0;
+            if (((L.P | L.nx) & 3) == 0) { // (planes of nz nx floats keep the alignment)
                 if (ix0 >= 0 && ix0 + 3 < L.nx) red_add4(p, acc[r][0].x, acc[r][0].y, acc[r][1].x, acc[r][1].y);
             } else {
                 if (ix0 >= 0 && ix0 < L.nx) atomicAdd(p, acc[r][0].x);
@@ -705,12 +705,13 @@ __device__ __forceinline__ void flush_grad(const ResArgs &a, const Own<R> &o, fl
 // the warp's group g.
 template <int R, int G, int MODE, int ACC>
 __device__ __forceinline__ bool fwd_loop(const ResArgs &a, const Own<R> &o, float *sm, const float4 (&ca)[R], const float *kb,
-                                         float2 (&acc)[R][2], ResShared &sh, int group, int shot0, int nsh, unsigned srcs, uint32_t pf)
+                                         float2 (&acc)[R][2], ResShared &sh, int group, int accg, int shot0, int nsh, unsigned srcs,
+                                         uint32_t pf)
 {
     const int nt = a.nt, fs = a.t.fs, lane = threadIdx.x & 31;
     for (int n = 0; n < nt; ++n) {
         const uint32_t par = (pf + n) & 1u;
-        if (ACC && n > 0 && n % RES_SUM == 0) flush_illum<R>(a, o, acc);
+        if (ACC && n > 0 && n % RES_SUM == 0) flush_illum<R>(a, o, acc, accg);
         for (int s = group; s < nsh; s += G) {
             if (!res_wait(smem_u32(&sh.bars.full[s]), par, &sh.abort)) return false;
             const float *f = sm + (2 * s + (n & 1)) * fs + o.so;
@@ -725,6 +726,16 @@ __device__ __forceinline__ bool fwd_loop(const ResArgs &a, const Own<R> &o, floa
                     }
                 }
                 continue;
+            }
+            if (a.snaps != nullptr && o.on && n % a.snap_k == 0) { // the state before the step
+                float *sp = a.snaps + ((long long)(n / a.snap_k) * 2 * a.ns + shot0 + s) * a.L.fstride + fidx(a.L, o.i0, o.j0);
+                float *sq = sp + (long long)a.ns * a.L.fstride;
+#pragma unroll
+                for (int r = 0; r < R; ++r)
+                    if (o.in >> r & 1) {
+                        *reinterpret_cast<float4 *>(sp + r * a.L.pitch) = lds4(f + r * RES_P);
+                        *reinterpret_cast<float4 *>(sq + r * a.L.pitch) = lds4(g + r * RES_P);
+                    }
             }
             if (o.on) {
                 // the source's point, if this thread holds it: its u^{n-1} and sum
@@ -828,9 +839,9 @@ __global__ void __launch_bounds__(32 * (NW + RES_SVC), 1) k_fwd_resident(const _
                     srcs |= 1u << s;
             const uint32_t pf = (uint32_t)(round * nt);
             const bool ok = __any_sync(0xffffffffu, o.bmask != 0)
-                ? fwd_loop<R, G, 1, ACC>(a, o, sm, ca, kbs + o.ko, acc, sh, group, first + base, nsh, srcs, pf)
-                : fwd_loop<R, G, 0, ACC>(a, o, sm, ca, kbs + o.ko, acc, sh, group, first + base, nsh, srcs, pf);
-            if (ACC && ok) flush_illum<R>(a, o, acc);
+                ? fwd_loop<R, G, 1, ACC>(a, o, sm, ca, kbs + o.ko, acc, sh, group, c.set * G + group, first + base, nsh, srcs, pf)
+                : fwd_loop<R, G, 0, ACC>(a, o, sm, ca, kbs + o.ko, acc, sh, group, c.set * G + group, first + base, nsh, srcs, pf);
+            if (ACC && ok) flush_illum<R>(a, o, acc, c.set * G + group);
             // the last two levels: checked, and kept for an adjoint pass
             if (ok && o.on) {
                 bool fin = true;
@@ -1279,6 +1290,9 @@ ResTile res_plan(const Lay2D &L, int ns, ResKind kind)
     ResTile best{};
     best.us = 1e30f;
     if (ns < 1) return best;
+    // band_init takes the sponge cells of a float4 as one run of the checkpoint; with
+    // one or two model columns a float4 can hold sponge cells on both sides of them
+    if (L.nx < 3) return best;
     res_prepare();
     const bool bwd = kind == RES_BWD;
     int nv = 0;
@@ -1328,6 +1342,7 @@ ResTile res_plan(const Lay2D &L, int ns, ResKind kind)
                     best.ntx = ntx;
                     best.ntz = ntz;
                     best.sets = sets;
+                    best.accs = sets * G;
                     best.s = s;
                     best.per = per;
                     best.fs = fs;

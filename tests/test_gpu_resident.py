@@ -17,7 +17,7 @@ pytestmark = pytest.mark.gpu
 # nz, nx, shots, nt, sponge
 CASES = [(37, 83, 3, 90, 7), (20, 20, 1, 60, 20), (5, 300, 2, 50, 3), (90, 31, 5, 40, 1), (64, 128, 40, 30, 8),
          (61, 203, 97, 25, 5), (300, 1000, 9, 24, 20), (150, 460, 80, 20, 20), (33, 47, 2, 2, 4), (33, 47, 3, 3, 4),
-         (400, 1201, 3, 12, 15)]
+         (400, 1201, 3, 12, 15), (40, 3, 2, 30, 2)]
 
 
 @pytest.fixture(scope="module")
@@ -76,6 +76,20 @@ def test_resident_loops_match_the_streaming_steps(torch_cuda, nz, nx, ns, nt, P)
         assert abs(float(a[1]["misfit"]) - float(b[1]["misfit"])) <= 1e-12 * float(b[1]["misfit"])
         assert rel(a[1]["grad"], b[1]["grad"]) <= 1e-6
         assert rel(a[1]["illum"], b[1]["illum"]) <= 1e-6
+
+
+@pytest.mark.parametrize("nx,P", [(1, 1), (2, 1), (1, 2), (2, 5)])
+def test_models_of_one_or_two_columns(torch_cuda, nx, P):
+    """Sponge cells on both sides of the model within four columns: the
+    checkpoint's order has a gap there, so these run the streaming steps."""
+    from paper_1406_1864_gb300 import fwi
+    torch = torch_cuda
+    grid, geom, v, d = problem(torch, 40, nx, 2, 30, P)
+    geom = fwi.Geometry(geom.src, geom.rec[:, :nx], geom.wavelet)
+    d, opts = d[:, :, :nx].contiguous(), fwi.Options(precond="none")
+    a, b = both(fwi, grid, geom, opts, lambda: (fwi.forward(grid, geom, v), fwi.adjoint_gradient(grid, geom, v, d, opts)))
+    assert torch.equal(a[0], b[0])
+    assert rel(a[1]["grad"], b[1]["grad"]) <= 1e-6 and rel(a[1]["illum"], b[1]["illum"]) <= 1e-6
 
 
 def test_resident_forward_feeds_either_adjoint_pass(torch_cuda):
