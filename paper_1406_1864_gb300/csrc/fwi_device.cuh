@@ -183,6 +183,30 @@ __device__ __forceinline__ void tma_load_3d(uint32_t dst, const CUtensorMap *map
                  : "memory");
 }
 
+// ---- overlap of a time loop's consecutive launches (programmatic dependent
+// launch). A step kernel lets the next one launch as soon as it has started
+// itself: the next kernel's CTAs then take the slots of those that have run out of
+// work, set up their barriers and work lists (which no step writes), and wait
+// in pdl_wait() until the step before has completed and its memory is visible.
+// Everything a step writes is read after that wait.
+__device__ __forceinline__ void pdl_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+__device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+
+inline cudaError_t launch_pdl(const void *fn, unsigned ctas, unsigned threads, size_t smem, void **params, cudaStream_t st)
+{
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(ctas);
+    cfg.blockDim = dim3(threads);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = st;
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = at;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelExC(&cfg, fn, params);
+}
+
 constexpr int align128(int b) { return (b + 127) / 128 * 128; }
 
 // shared-memory plan of a step kernel: mbarriers, then STAGES stages of

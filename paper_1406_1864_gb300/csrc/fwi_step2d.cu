@@ -74,15 +74,13 @@ struct alignas(16) ItemDesc {
 // State of the staging lane that walks the CTA's chunks.
 struct Cursor {
     int model, tile, s, s_end; // current chunk
-    int q_next;                // next chunk, taken one chunk ahead (-1: none)
     bool done;
 };
 
-__device__ __forceinline__ int grab_chunk(int *counter, int nchunks)
-{
-    const int q = atomicAdd(counter, 1);
-    return q < nchunks ? q : -1;
-}
+// the first chunk of a CTA is its index (no atomic before the first copies), the
+// counter hands out those after the grid's. The staging lane keeps the answer
+// in a register until it needs it, a chunk later: nothing waits for the atomic.
+__device__ __forceinline__ int grab_chunk(int *counter) { return (int)gridDim.x + atomicAdd(counter, 1); }
 
 // chunk q of a launch: its model (chunks of the models are consecutive),
 // tile and shot range
@@ -114,32 +112,32 @@ __device__ __forceinline__ void cursor_set(Cursor &cu, int q, const BT &B)
 }
 
 template <class BT>
-__device__ __forceinline__ void cursor_init(Cursor &cu, const BT &B)
+__device__ __forceinline__ void cursor_init(Cursor &cu, int &q_next, const BT &B)
 {
     const int nchunks = B.chunk_end[B.nm - 1];
-    const int q = grab_chunk(B.sched, nchunks);
+    const int q = (int)blockIdx.x < nchunks ? (int)blockIdx.x : -1;
     cu.done = q < 0;
-    cu.q_next = -1;
+    q_next = -1;
     cu.model = cu.tile = cu.s = cu.s_end = 0;
     if (!cu.done) {
         cursor_set(cu, q, B);
-        cu.q_next = grab_chunk(B.sched, nchunks);
+        q_next = grab_chunk(B.sched);
     }
 }
 
 // next (model, tile, shots s .. s + cnt - 1 with cnt <= spi) of this CTA;
 // false when the launch's work is exhausted
 template <class BT>
-__device__ __forceinline__ bool cursor_next(Cursor &cu, const BT &B, int &model, int &tile, int &s, int spi, int &cnt)
+__device__ __forceinline__ bool cursor_next(Cursor &cu, int &q_next, const BT &B, int &model, int &tile, int &s, int spi, int &cnt)
 {
     if (cu.done) return false;
     if (cu.s >= cu.s_end) {
-        if (cu.q_next < 0) {
+        if (q_next >= B.chunk_end[B.nm - 1]) {
             cu.done = true;
             return false;
         }
-        cursor_set(cu, cu.q_next, B);
-        cu.q_next = grab_chunk(B.sched, B.chunk_end[B.nm - 1]);
+        cursor_set(cu, q_next, B);
+        q_next = grab_chunk(B.sched);
     }
     model = cu.model;
     tile = cu.tile;
@@ -171,10 +169,10 @@ __device__ __forceinline__ bool has_rec(const BornArgs &a) { return a.dseis != n
 // staging thread calls before the barrier that publishes the slot. The
 // amplitude is stored unscaled (times src_scale at use).
 template <int SPI, class BT>
-__device__ __forceinline__ void stage_desc_async(ItemDesc *slot, Cursor &cu, const BT &B, int n_src, bool use_src)
+__device__ __forceinline__ void stage_desc_async(ItemDesc *slot, Cursor &cu, int &q_next, const BT &B, int n_src, bool use_src)
 {
     int mdl = 0, t = -1, s = 0, cnt = 0;
-    if (!cursor_next(cu, B, mdl, t, s, SPI, cnt)) t = -1;
+    if (!cursor_next(cu, q_next, B, mdl, t, s, SPI, cnt)) t = -1;
     slot->tile = t;
     slot->s = s;
     slot->model = mdl;
@@ -360,6 +358,7 @@ __global__ void __launch_bounds__(TPB, MINB) k_fwd_step(const __grid_constant__ 
     const FwdArgs &a0 = B.m[0];
     const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
 
+    pdl_trigger();
     if (threadIdx.x == 0) {
         for (int k = 0; k < STAGES; ++k) mbar_init(smem_u32(&bars[k]), 1);
         fence_mbar_init();
@@ -370,7 +369,8 @@ __global__ void __launch_bounds__(TPB, MINB) k_fwd_step(const __grid_constant__ 
     // lane 0 of warp 1 walks the chunks (cursor in shared memory) and stages
     // descriptors D + 1 items ahead
     __shared__ Cursor s_cu;
-    auto stage = [&](int slot) { stage_desc_async<SPI>(&s_desc[slot % DESC_RING], s_cu, B, a0.n, !a0.last); };
+    int q_next = -1; // next chunk (staging lane), taken one chunk ahead
+    auto stage = [&](int slot) { stage_desc_async<SPI>(&s_desc[slot % DESC_RING], s_cu, q_next, B, a0.n, !a0.last); };
     auto issue = [&](const ItemDesc &d, int k) {
         const FwdArgs &ad = B.m[NM == 1 ? 0 : d.model];
         const int bz = d.tile / ad.c.ntx, bx = d.tile - bz * ad.c.ntx;
@@ -385,11 +385,12 @@ __global__ void __launch_bounds__(TPB, MINB) k_fwd_step(const __grid_constant__ 
     // lane 0 of warp 1 walks the chunks and stages descriptors; thread 0
     // issues the copies of a descriptor staged one barrier earlier
     if (threadIdx.x == 32) {
-        cursor_init(s_cu, B);
+        cursor_init(s_cu, q_next, B);
         for (int k = 0; k <= D; ++k) stage(k);
         cp_async_wait_all();
     }
     __syncthreads();
+    pdl_wait();
     if (threadIdx.x == 0)
         for (int k = 0; k < D; ++k)
             if (s_desc[k].tile >= 0) issue(s_desc[k], k);
@@ -785,6 +786,7 @@ __global__ void __launch_bounds__(TPB, MINB) k_bwd_step(const __grid_constant__ 
     const bool recon = a0.recon != 0;
     const bool need_band = recon && m >= 3; // u^{m-2} in the sponge comes from checkpoint m-2 >= 1
 
+    pdl_trigger();
     if (threadIdx.x == 0) {
         for (int k = 0; k < STAGES; ++k) mbar_init(smem_u32(&bars[k]), 1);
         fence_mbar_init();
@@ -794,7 +796,8 @@ __global__ void __launch_bounds__(TPB, MINB) k_bwd_step(const __grid_constant__ 
     __syncthreads();
 
     __shared__ Cursor s_cu;
-    auto stage = [&](int slot) { stage_desc_async<1>(&s_desc[slot % DESC_RING], s_cu, B, m - 1, true); };
+    int q_next = -1; // next chunk (staging lane), taken one chunk ahead
+    auto stage = [&](int slot) { stage_desc_async<1>(&s_desc[slot % DESC_RING], s_cu, q_next, B, m - 1, true); };
     auto issue = [&](const ItemDesc &d, int k) {
         const BwdArgs &a = B.m[NM == 1 ? 0 : d.model];
         const int bz = d.tile / a.c.ntx, bx = d.tile - bz * a.c.ntx;
@@ -815,11 +818,12 @@ __global__ void __launch_bounds__(TPB, MINB) k_bwd_step(const __grid_constant__ 
     // lane 0 of warp 1 walks the chunks and stages descriptors; thread 0
     // issues the copies of a descriptor staged one barrier earlier
     if (threadIdx.x == 32) {
-        cursor_init(s_cu, B);
+        cursor_init(s_cu, q_next, B);
         for (int k = 0; k <= D; ++k) stage(k);
         cp_async_wait_all();
     }
     __syncthreads();
+    pdl_wait();
     if (threadIdx.x == 0)
         for (int k = 0; k < D; ++k)
             if (s_desc[k].tile >= 0) issue(s_desc[k], k);
@@ -1159,6 +1163,7 @@ __global__ void __launch_bounds__(TPB, MINB) k_born_step(const __grid_constant__
     const Lay2D &L = c.L;
     const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
 
+    pdl_trigger();
     if (threadIdx.x == 0) {
         for (int k = 0; k < STAGES; ++k) mbar_init(smem_u32(&bars[k]), 1);
         fence_mbar_init();
@@ -1166,7 +1171,8 @@ __global__ void __launch_bounds__(TPB, MINB) k_born_step(const __grid_constant__
     }
     __syncthreads();
 
-    auto stage = [&](int slot) { stage_desc_async<1>(&s_desc[slot % DESC_RING], s_cu, B, a.n, !a.last); };
+    int q_next = -1; // next chunk (staging lane), taken one chunk ahead
+    auto stage = [&](int slot) { stage_desc_async<1>(&s_desc[slot % DESC_RING], s_cu, q_next, B, a.n, !a.last); };
     auto issue = [&](const ItemDesc &d, int k) {
         const int bz = d.tile / c.ntx, bx = d.tile - bz * c.ntx;
         const int bi = bz * TZ, bj = bx * TX;
@@ -1182,11 +1188,12 @@ __global__ void __launch_bounds__(TPB, MINB) k_born_step(const __grid_constant__
         }
     };
     if (threadIdx.x == 32) {
-        cursor_init(s_cu, B);
+        cursor_init(s_cu, q_next, B);
         for (int k = 0; k <= D; ++k) stage(k);
         cp_async_wait_all();
     }
     __syncthreads();
+    pdl_wait();
     if (threadIdx.x == 0)
         for (int k = 0; k < D; ++k)
             if (s_desc[k].tile >= 0) issue(s_desc[k], k);
@@ -1489,6 +1496,8 @@ __global__ void __launch_bounds__(TPB, 4) k_offh_level(const float *__restrict__
         }
     };
     const int nstage = (nsh + SPS - 1) / SPS;
+    pdl_trigger();
+    pdl_wait();
 #pragma unroll
     for (int k = 0; k < NST - 1; ++k) {
         if (k < nstage) stage(k, k);
@@ -1693,7 +1702,7 @@ cudaError_t launch_variant(const Variant &v, int b, Batch<A, N> &args, int ctas,
 {
     if (ctas <= 0) return cudaSuccess;
     void *params[] = {&args};
-    return cudaLaunchKernel(v.fn[b], dim3(ctas), dim3(TPB), params, (size_t)v.smem, st);
+    return launch_pdl(v.fn[b], ctas, TPB, (size_t)v.smem, params, st);
 }
 } // namespace
 
@@ -1808,11 +1817,13 @@ cudaError_t launch_offh_sums(const FwdArgs &a, cudaStream_t st)
     const int nch = std::max(1, std::min(ns, sm_count_dev() * occ / std::max(1, ntiles)));
     const int chunk = ((ns + nch - 1) / nch + 1) & ~1;
     const int grid = ntiles * ((ns + chunk - 1) / chunk);
-    if (a.hmax <= 10)
-        k_offh_level<11, 3, 4><<<grid, TPB, 0, st>>>(a.uin, L, ns, chunk, a.hmax, a.acc_offh);
-    else
-        k_offh_level<13, 3, 4><<<grid, TPB, 0, st>>>(a.uin, L, ns, chunk, a.hmax, a.acc_offh);
-    return cudaGetLastError();
+    const float *uin = a.uin;
+    Lay2D lay = L;
+    int n = ns, ck = chunk, hm = a.hmax;
+    float *acc = a.acc_offh;
+    void *params[] = {&uin, &lay, &n, &ck, &hm, &acc};
+    const void *fn = a.hmax <= 10 ? (const void *)k_offh_level<11, 3, 4> : (const void *)k_offh_level<13, 3, 4>;
+    return launch_pdl(fn, grid, TPB, 0, params, st);
 }
 } // namespace
 
@@ -1897,8 +1908,8 @@ template <int HE> struct ExtKernels {
         Batch<BwdArgs, 1> b;
         const int ctas = batch_fill(b, &a, &t, 1, occ_b);
         if (ctas <= 0) return cudaSuccess;
-        k_bwd_step<1, 2, 3, 1, HE><<<ctas, TPB, SMEM_B, st>>>(b);
-        return cudaGetLastError();
+        void *params[] = {&b};
+        return launch_pdl((const void *)k_bwd_step<1, 2, 3, 1, HE>, ctas, TPB, SMEM_B, params, st);
     }
     static cudaError_t born(const BornArgs &a, const Tiling &t, cudaStream_t st)
     {
@@ -1906,8 +1917,8 @@ template <int HE> struct ExtKernels {
         Batch<BornArgs, 1> b;
         const int ctas = batch_fill(b, &a, &t, 1, occ_o);
         if (ctas <= 0) return cudaSuccess;
-        k_born_step<1, 2, 3, HE><<<ctas, TPB, SMEM_O, st>>>(b);
-        return cudaGetLastError();
+        void *params[] = {&b};
+        return launch_pdl((const void *)k_born_step<1, 2, 3, HE>, ctas, TPB, SMEM_O, params, st);
     }
 };
 template <int HE> std::once_flag ExtKernels<HE>::once;
@@ -1960,8 +1971,8 @@ cudaError_t launch_born_step(const BornArgs &a, const Tiling &t, cudaStream_t st
     Batch<BornArgs, 1> b;
     const int ctas = batch_fill(b, &a, &t, 1, g_occ_born);
     if (ctas <= 0) return cudaSuccess;
-    K_BORN<<<ctas, TPB, SMEM_BORN, st>>>(b);
-    return cudaGetLastError();
+    void *params[] = {&b};
+    return launch_pdl((const void *)K_BORN, ctas, TPB, SMEM_BORN, params, st);
 }
 
 // Tensor map over `nfields` stored fields [nfields][rows][pitch] (float32)

@@ -146,6 +146,7 @@ __global__ void __launch_bounds__(TPB, MINB) k_fwd3d(const __grid_constant__ Fwd
     const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
     const int ntiles = c.nty * c.ntx;
 
+    pdl_trigger();
     if (threadIdx.x == 0) {
         for (int k = 0; k < STAGES; ++k) mbar_init(smem_u32(&bars[k]), 1);
         fence_mbar_init();
@@ -187,6 +188,7 @@ __global__ void __launch_bounds__(TPB, MINB) k_fwd3d(const __grid_constant__ Fwd
         tma_load_4d(smem_u32(sg + HALO3 + 2 * PT3), &a.tm_c2, GXL + bj, bk + GY, i + GZ, 0, bar);
         tma_load_4d(smem_u32(sg + HALO3 + 3 * PT3), &a.tm_damp, GXL + bj, bk + GY, i + GZ, 0, bar);
     };
+    pdl_wait();
     if (threadIdx.x == 0)
         for (int t = 0; t < D; ++t) issue(t);
     __syncthreads();
@@ -343,6 +345,7 @@ __global__ void __launch_bounds__(TPB, MINB) k_bwd3d(const __grid_constant__ Bwd
     const int ntiles = c.nty * c.ntx;
     const int m = a.m;
 
+    pdl_trigger();
     if (threadIdx.x == 0) {
         for (int k = 0; k < STAGES; ++k) mbar_init(smem_u32(&bars[k]), 1);
         fence_mbar_init();
@@ -384,6 +387,7 @@ __global__ void __launch_bounds__(TPB, MINB) k_bwd3d(const __grid_constant__ Bwd
         tma_load_4d(smem_u32(sg + HALO3 + 3 * PT3), &a.tm_damp, GXL + bj, bk + GY, i + GZ, 0, bar);
         tma_load_4d(smem_u32(sg + HALO3 + 4 * PT3), &a.tm_q, GXL + bj, bk + GY, i + GZ, iss.s, bar);
     };
+    pdl_wait();
     if (threadIdx.x == 0)
         for (int t = 0; t < D; ++t) issue(t);
     __syncthreads();
@@ -769,7 +773,7 @@ cudaError_t launch3(const void *fn, const Variant3 &v, const A &a, const Tiling3
 {
     if (t.ctas <= 0) return cudaSuccess;
     void *args[] = {const_cast<A *>(&a)};
-    return cudaLaunchKernel(fn, dim3(t.ctas), dim3(TPB), args, v.smem, st);
+    return launch_pdl(fn, t.ctas, TPB, v.smem, args, st);
 }
 } // namespace
 
