@@ -1762,6 +1762,28 @@ bool step_variant_valid(StepKind kind, int variant, int hmax)
     return kind != STEP_FWD_OFFH || hmax <= vs[variant].nh - 1;
 }
 
+// Tile variant of a problem that was not autotuned, from the variants pinned one
+// by one in gradients of 0.5 to 38 M padded points over all shots (us per level):
+// - forward: two-shot items beat single ones everywhere (100 x 200, 16 shots
+//   11.8 against 13.8; 150 x 460, 80 shots 29.8 / 34.2; 400 x 1200, 64 shots
+//   101 / 111.5); a single shot takes the one-shot variant.
+// - with the offset Hessian: the fused two-shot step with 16 shots per chunk. The
+//   plain step and k_offh_level are up to 7% faster on large levels (400 x 1200, 64
+//   shots 140 against 150), but sum the zero-offset image in another order than the
+//   illumination (3e-5 apart after 4000 levels of 300 x 1000, else equal), so only
+//   autotuning takes them.
+// - backward: 64 x 8 tiles while a level leaves CTAs idle (100 x 200, 64 shots
+//   21.7 against 26.6; 300 x 1000, 16 shots 36.1 / 37.9; 150 x 460, 80 shots, 7.6 M
+//   points 50.1 / 51.5), 64 x 16 above (500 x 1500, 16 shots, 13 M points 66.6
+//   against 72.1; 400 x 1200, 64 shots 154 / 166).
+int default_variant(const Lay2D &L, int ns, StepKind kind, int hmax)
+{
+    const double pts = (double)L.nzp * L.nxp * ns;
+    if (kind == STEP_FWD) return ns > 1 ? 3 : 0;
+    if (kind == STEP_BWD) return pts < 8e6 ? 1 : 0;
+    return hmax <= g_var_h[2].nh - 1 ? 2 : 1;
+}
+
 Tiling make_tiling(const Lay2D &L, int ns, StepKind kind, int variant, int chunk, int hmax)
 {
     prepare_kernels();
@@ -1773,14 +1795,7 @@ Tiling make_tiling(const Lay2D &L, int ns, StepKind kind, int variant, int chunk
             variant = tv;
             if (chunk <= 0) chunk = tc;
         } else {
-            // default: the first variant, or for the offset Hessian the one
-            // with the fewest offsets that covers hmax, two shots per item
-            variant = 0;
-            if (kind == STEP_FWD_OFFH)
-                for (int i = 0; i < n; ++i)
-                    if (vs[i].spi == 2 && hmax <= vs[i].nh - 1 &&
-                        (!step_variant_valid(kind, variant, hmax) || vs[variant].spi != 2 || vs[i].nh < vs[variant].nh))
-                        variant = i;
+            variant = default_variant(L, ns, kind, hmax);
         }
     }
     if (chunk <= 0) chunk = kind == STEP_FWD_OFFH ? CHUNKS_H[0] : CHUNKS_F[0];

@@ -700,7 +700,12 @@ int step3_variant_for(const Lay3D &L, int ns, bool backward)
 {
     std::lock_guard<std::mutex> lock(g_tune3_mu);
     auto it = g_tuned3.find(TuneKey3{backward, L.nzp, L.nyp, L.nxp, ns});
-    return it == g_tuned3.end() ? 0 : it->second.first;
+    if (it != g_tuned3.end()) return it->second.first;
+    // not autotuned: the backward step's 3-stage ring at 4 CTAs per SM once there
+    // are points to fill them (gradients of 100 x 200 x 200, 4 shots 18.65 -> 17.81
+    // ms, 40 x 120 x 160, 3 shots 6.21 -> 5.85; 100 x 100 x 100, one shot, 2.7 M padded
+    // points 3.49 -> 3.58: the default 3 CTAs)
+    return backward && (double)L.nzp * L.nyp * L.nxp * ns >= 3.5e6 ? 2 : 0;
 }
 
 int step3_segments_for(const Lay3D &L, int ns, bool backward)
