@@ -217,13 +217,14 @@ bool receivers_fit(const Lay2D &L, const fwi_geometry *ge, const ResTile &t, boo
     return true;
 }
 
-// Level of the streaming steps in us, fitted to the measured ones (recorded
-// graphs, autotuned tiles) from 0.1 M to 34 M padded points: forward 7.1, 22.6,
-// 27.3 and 84 us at 0.13, 4.2, 7.6 and 34 M; backward 9.2, 34, 51 and 157 us.
+// Level of the streaming steps in us, fitted to the measured ones from 0.1 M to
+// 17 M padded points: forward 7.1, 14.9, 15.7, 23.4 and 29.8 us at 0.13, 2.2, 3.4,
+// 5.7 and 7.6 M; backward 9.2, 21.7, 26.8, 36.1, 50.1 and 87 us at 0.13, 2.2, 3.4,
+// 5.7, 7.6 and 17 M.
 double streaming_us(double pts, ResKind kind)
 {
-    return kind == RES_BWD ? std::min(8.0 + 9e-6 * pts, 20.0 + 4.0e-6 * pts)
-                           : std::min(6.0 + 4.0e-6 * pts, 14.0 + 2.0e-6 * pts);
+    return kind == RES_BWD ? std::min(8.0 + 9e-6 * pts, 11.0 + 4.8e-6 * pts)
+                           : std::min(6.0 + 4.0e-6 * pts, 9.0 + 2.6e-6 * pts);
 }
 
 // The levels that a resident forward pass keeps for the offset-Hessian sums
@@ -805,6 +806,8 @@ fwi_status run_forward_models(int nm, const Plan *pl, const fwi_geometry *const 
             a[k].uin = U[k][n & 1];
             a[k].uout = U[k][(n + 1) & 1];
         }
+        // (the levels' launches overlap, see pdl_wait: 400 x 1200, 64 shots 93.0 ->
+        // 89.8 us per level, Gauss-Newton products of 300 x 1000, 48 shots 176 -> 170)
         e = nm == 1 ? launch_fwd_step(a[0], til[0], offh, st) : launch_fwd_batch(a.data(), til.data(), nm, offh, st);
         if (e != cudaSuccess) return cuda_fail(e, "forward step");
         t_launch[0] += fwd_split(til[0], offh) ? 1 + nm : 1; // (split: one offset-Hessian sum per model)
