@@ -188,8 +188,11 @@ Lay2D make_layout(const fwi_grid *g)
     L.pitch = (int)align_up((size_t)(GXL + L.nxp + GXR), 32);
     L.rows = L.nzp + 2 * GZ;
     L.fstride = (long long)align_up((size_t)L.rows * L.pitch, 64);
-    L.nband = 2 * L.P * L.nxp + 2 * L.P * L.nz;
-    L.nbandp = (L.nband + 3) / 4 * 4;
+    // (whole float4s of every row: forward passes that keep checkpoints, us per level,
+    // cells packed -> padded: 300 x 1001, 48 shots 72.0 -> 49.1, 200 x 401, 32 shots
+    // 27.3 -> 14.9, 71 x 333, 90 shots 29.2 -> 16.1; widths that are a multiple of 4
+    // 49.2 -> 48.3, 14.7 -> 14.7, 16.0 -> 15.7)
+    L.nbandp = band_size(L);
     L.dt = g->dt;
     L.dx = g->dx;
     const double etamax = 3.0 * g->vref * std::log(1.0 / g->refl) / (2.0 * g->sponge * g->dx);

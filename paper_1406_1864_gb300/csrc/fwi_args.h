@@ -36,8 +36,7 @@ struct Lay2D {
     int pitch;            // floats per stored row
     int rows;             // stored rows = nzp + 2 GZ
     long long fstride;    // floats per stored field (rows * pitch), 64-float aligned
-    int nband;            // sponge cells of one field (checkpointed each step)
-    int nbandp;           // per-step checkpoint stride: nband rounded up to 4 floats
+    int nbandp;           // slots of the per-step sponge checkpoint of one field
     float dt, dx;
     float etamax_dt;      // eta_max * dt
     float inv_p2;         // 1 / P^2
@@ -54,17 +53,37 @@ __host__ __device__ inline int sponge_depth(int i, int P, int n)
     return i < P ? P - i : (i >= P + n ? i - (P + n - 1) : 0);
 }
 
+// Slots per row of the sponge checkpoint: a top or bottom row; the left and the
+// right part of a model row. Rows and parts start on 16 bytes and the parts hold
+// whole float4s of the row (the few model cells among them have slots too), so
+// that the steps move 4 cells with one access whatever the width: with the cells
+// packed, widths that are no multiple of 4 took single 4-byte accesses on most
+// sponge rows.
+__host__ __device__ inline int band_row(const Lay2D &L) { return (L.nxp + 3) & ~3; }
+__host__ __device__ inline int band_left(const Lay2D &L) { return (L.P + 3) & ~3; }
+__host__ __device__ inline int band_right0(const Lay2D &L) // first column of the right part
+{
+    const int a = (L.P + L.nx) & ~3, b = band_left(L);
+    return a > b ? a : b;
+}
+__host__ __device__ inline int band_mid(const Lay2D &L)
+{
+    const int r = band_row(L) - band_right0(L);
+    return band_left(L) + (r > 0 ? r : 0);
+}
+__host__ __device__ inline int band_size(const Lay2D &L) { return 2 * L.P * band_row(L) + L.nz * band_mid(L); }
+
 // index of sponge cell (i, j) in the per-step checkpoint of one field;
-// -1 for model cells. Order: top P rows, then (left P, right P) per model row,
+// -1 for model cells. Order: top P rows, then (left, right) per model row,
 // then bottom P rows.
 __host__ __device__ inline int band_index(const Lay2D &L, int i, int j)
 {
-    const int P = L.P;
-    if (i < P) return i * L.nxp + j;
-    if (i >= P + L.nz) return P * L.nxp + 2 * P * L.nz + (i - P - L.nz) * L.nxp + j;
-    if (j < P) return P * L.nxp + (i - P) * 2 * P + j;
-    if (j >= P + L.nx) return P * L.nxp + (i - P) * 2 * P + P + (j - P - L.nx);
-    return -1;
+    const int P = L.P, w = band_row(L);
+    if (i < P) return i * w + j;
+    if (i >= P + L.nz) return P * w + L.nz * band_mid(L) + (i - P - L.nz) * w + j;
+    if (j >= P && j < P + L.nx) return -1;
+    const int row = P * w + (i - P) * band_mid(L), left = band_left(L);
+    return j < left ? row + j : row + left + j - band_right0(L);
 }
 
 // ------------------------------------------------------- receiver tables

@@ -1290,8 +1290,8 @@ ResTile res_plan(const Lay2D &L, int ns, ResKind kind)
     ResTile best{};
     best.us = 1e30f;
     if (ns < 1) return best;
-    // band_init takes the sponge cells of a float4 as one run of the checkpoint; with
-    // one or two model columns a float4 can hold sponge cells on both sides of them
+    // one or two model columns (sponge cells on both sides of them within four
+    // columns) are left to the streaming steps
     if (L.nx < 3) return best;
     res_prepare();
     const bool bwd = kind == RES_BWD;

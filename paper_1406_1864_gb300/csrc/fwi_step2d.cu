@@ -228,9 +228,9 @@ __device__ void abort_drain_ring(uint64_t *bars, const ItemDesc *desc, int k, in
         if (desc[j % DESC_RING].tile >= 0) mbar_wait(smem_u32(&bars[j % STAGES]), (j / STAGES) & 1, DRAIN_NS);
 }
 
-// Where the thread's float4 of each row sits in the per-step sponge
-// checkpoint: >= 0: checkpoint index of the 4 points (contiguous, 16-byte
-// aligned); -1: no sponge point; -2: mixed row (scalar path).
+// Where the thread's float4 of each row sits in the per-step sponge checkpoint
+// (contiguous, 16-byte aligned): >= 0: checkpoint index of 4 sponge points; -1: no
+// sponge point; below: some are sponge points, the index and a bit for each.
 template <int RZ>
 struct SpongeInfo {
     int brow[RZ];
@@ -241,28 +241,24 @@ struct SpongeInfo {
             const int i = i0 + r;
             int info = -1;
             if (i < L.nzp && j0 < L.nxp) {
-                bool any = false, all = true;
+                int mask = 0, base = 0;
 #pragma unroll
                 for (int p = 0; p < 4; ++p) {
-                    const bool inb = j0 + p < L.nxp && band_index(L, i, j0 + p) >= 0;
-                    any |= inb;
-                    all &= inb;
+                    const int b = j0 + p < L.nxp ? band_index(L, i, j0 + p) : -1;
+                    if (b >= 0) {
+                        mask |= 1 << p;
+                        base = b - p;
+                    }
                 }
-                if (any) {
-                    const int b0 = band_index(L, i, j0);
-                    info = (all && b0 >= 0 && band_index(L, i, j0 + 3) == b0 + 3 && (b0 & 3) == 0) ? b0 : -2;
-                }
+                if (mask != 0) info = mask == 15 ? base : -2 - (4 * base + mask);
             }
             brow[r] = info;
         }
     }
+    __device__ __forceinline__ bool any(int r) const { return brow[r] != -1; }
+    __device__ __forceinline__ int index(int r) const { return brow[r] >= 0 ? brow[r] : ((-2 - brow[r]) >> 2) & ~3; }
+    __device__ __forceinline__ int mask(int r) const { return brow[r] >= 0 ? 15 : (-2 - brow[r]) & 15; }
 };
-
-// sponge point (i, j) of the padded grid (inside the padded grid only)
-__device__ __forceinline__ bool in_band(const Lay2D &L, int i, int j)
-{
-    return i < L.nzp && j < L.nxp && band_index(L, i, j) >= 0;
-}
 
 // index (row * 4 + column) of the thread's point that holds the source, or -1
 template <int RZ>
@@ -575,15 +571,9 @@ __global__ void __launch_bounds__(TPB, MINB) k_fwd_step(const __grid_constant__ 
                         }
                         const float o[4] = {out[0].x, out[0].y, out[1].x, out[1].y};
                         if ((!QOUT || a.uout != nullptr) && colok && i < L.nzp) store4(up + fidx(L, i, j0), j0, L.nxp, o);
-                        if (a.band != nullptr && sg.brow[r] != -1) {
+                        if (a.band != nullptr && sg.any(r)) {
                             float *bb = a.band + ((long long)ss * c.nt + a.n + 1) * L.nbandp;
-                            if (sg.brow[r] >= 0) {
-                                *reinterpret_cast<float4 *>(bb + sg.brow[r]) = make_float4(o[0], o[1], o[2], o[3]);
-                            } else {
-#pragma unroll
-                                for (int p = 0; p < 4; ++p)
-                                    if (in_band(L, i, j0 + p)) bb[band_index(L, i, j0 + p)] = o[p];
-                            }
+                            *reinterpret_cast<float4 *>(bb + sg.index(r)) = make_float4(o[0], o[1], o[2], o[3]);
                         }
                     }
                     if (a.illum_utt) {
@@ -889,18 +879,9 @@ __global__ void __launch_bounds__(TPB, MINB) k_bwd_step(const __grid_constant__ 
 #pragma unroll
         for (int r = 0; r < RZ; ++r) {
             bv[r] = make_float4(0.f, 0.f, 0.f, 0.f);
-            if (need_band && sg.brow[r] != -1) {
+            if (need_band && sg.any(r)) {
                 const float *bb = a.band + ((long long)s * c.nt + (m - 2)) * L.nbandp;
-                if (sg.brow[r] >= 0) {
-                    bv[r] = __ldcs(reinterpret_cast<const float4 *>(bb + sg.brow[r]));
-                } else {
-                    const int i = i0 + r;
-                    float t[4] = {0.f, 0.f, 0.f, 0.f};
-#pragma unroll
-                    for (int p = 0; p < 4; ++p)
-                        if (in_band(L, i, j0 + p)) t[p] = __ldcs(bb + band_index(L, i, j0 + p));
-                    bv[r] = make_float4(t[0], t[1], t[2], t[3]);
-                }
+                bv[r] = __ldcs(reinterpret_cast<const float4 *>(bb + sg.index(r)));
             }
         }
     };
@@ -1089,10 +1070,10 @@ __global__ void __launch_bounds__(TPB, MINB) k_bwd_step(const __grid_constant__ 
                     float unew[4] = {un[0].x, un[0].y, un[1].x, un[1].y};
                     if (sg.brow[r] >= 0) {
                         unew[0] = bnow[r].x; unew[1] = bnow[r].y; unew[2] = bnow[r].z; unew[3] = bnow[r].w;
-                    } else if (sg.brow[r] == -2) {
+                    } else if (sg.any(r)) {
 #pragma unroll
                         for (int p = 0; p < 4; ++p)
-                            if (in_band(L, i, j0 + p)) unew[p] = comp(bnow[r], p);
+                            if (sg.mask(r) >> p & 1) unew[p] = comp(bnow[r], p);
                     }
                     if (colok && i < L.nzp) {
                         store4(a.pb + so + fidx(L, i, j0), j0, L.nxp, pnew);
@@ -1367,15 +1348,9 @@ __global__ void __launch_bounds__(TPB, MINB) k_born_step(const __grid_constant__
                         const float dox[4] = {dn[0].x, dn[0].y, dn[1].x, dn[1].y};
                         store4(a.uout + so + fidx(L, i, j0), j0, L.nxp, uo);
                         store4(a.duout + so + fidx(L, i, j0), j0, L.nxp, dox);
-                        if (tile_sponge && a.band != nullptr && sg.brow[r] != -1) {
+                        if (tile_sponge && a.band != nullptr && sg.any(r)) {
                             float *bb = a.band + ((long long)s * c.nt + a.n + 1) * L.nbandp;
-                            if (sg.brow[r] >= 0) {
-                                *reinterpret_cast<float4 *>(bb + sg.brow[r]) = make_float4(uo[0], uo[1], uo[2], uo[3]);
-                            } else {
-#pragma unroll
-                                for (int p = 0; p < 4; ++p)
-                                    if (in_band(L, i, j0 + p)) bb[band_index(L, i, j0 + p)] = uo[p];
-                            }
+                            *reinterpret_cast<float4 *>(bb + sg.index(r)) = make_float4(uo[0], uo[1], uo[2], uo[3]);
                         }
                     }
                 }

@@ -80,8 +80,8 @@ def test_resident_loops_match_the_streaming_steps(torch_cuda, nz, nx, ns, nt, P)
 
 @pytest.mark.parametrize("nx,P", [(1, 1), (2, 1), (1, 2), (2, 5)])
 def test_models_of_one_or_two_columns(torch_cuda, nx, P):
-    """Sponge cells on both sides of the model within four columns: the
-    checkpoint's order has a gap there, so these run the streaming steps."""
+    """Sponge cells on both sides of the model within four columns: these run
+    the streaming steps."""
     from paper_1406_1864_gb300 import fwi
     torch = torch_cuda
     grid, geom, v, d = problem(torch, 40, nx, 2, 30, P)
