@@ -1747,15 +1747,24 @@ bool step_variant_valid(StepKind kind, int variant, int hmax)
 //   shots 140 against 150), but sum the zero-offset image in another order than the
 //   illumination (3e-5 apart after 4000 levels of 300 x 1000, else equal), so only
 //   autotuning takes them.
-// - backward: 64 x 8 tiles while a level leaves CTAs idle (100 x 200, 64 shots
-//   21.7 against 26.6; 300 x 1000, 16 shots 36.1 / 37.9; 150 x 460, 80 shots, 7.6 M
-//   points 50.1 / 51.5), 64 x 16 above (500 x 1500, 16 shots, 13 M points 66.6
-//   against 72.1; 400 x 1200, 64 shots 154 / 166).
+// - backward: the variant with the shorter level by rounds of resident CTAs; a
+//   round of 64 x 8 tiles (5 CTAs per SM) takes about 0.75 of one of 64 x 16 (4 per
+//   SM): 15 against 20 us at 8 shots per chunk. One round each: 100 x 200, 64 shots
+//   21.7 against 26.6, 300 x 1000, 2 shots 7.3 / 8.8; two against one: 71 x 332, 90
+//   shots 37.8 / 27.1, 200 x 400, 32 shots 29.0 / 26.1; two each: 300 x 1000, 16 shots
+//   36.1 / 37.9; many: 500 x 1500, 16 shots 72.1 / 66.6, 400 x 1200, 64 shots 166 / 154.
 int default_variant(const Lay2D &L, int ns, StepKind kind, int hmax)
 {
-    const double pts = (double)L.nzp * L.nxp * ns;
     if (kind == STEP_FWD) return ns > 1 ? 3 : 0;
-    if (kind == STEP_BWD) return pts < 8e6 ? 1 : 0;
+    if (kind == STEP_BWD) {
+        auto rounds = [&](const Variant &v) {
+            const long long tiles = (long long)((L.nxp + TX - 1) / TX) * ((L.nzp + 8 * v.rz - 1) / (8 * v.rz));
+            const long long slots = std::max(1LL, (long long)sm_count_dev() * v.occ[0]);
+            const int chunk = std::min(ns, CHUNKS_F[0]);
+            return (tiles * chunk_blocks(ns, chunk) + slots - 1) / slots;
+        };
+        return 3 * rounds(g_var_b[1]) < 4 * rounds(g_var_b[0]) ? 1 : 0;
+    }
     return hmax <= g_var_h[2].nh - 1 ? 2 : 1;
 }
 
