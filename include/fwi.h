@@ -354,7 +354,11 @@ fwi_status fwi_gauss_newton_hvp(const fwi_grid *grid, const fwi_geometry *geom, 
    plans of the same shape use them (a batch uses model 0's). choice: NULL
    or int[4] = forward variant, forward chunk, backward variant, backward
    chunk. The timing leaves ws in an unspecified state (the next call's
-   set-up rewrites it). fwi_autotune_reset() forgets all choices.
+   set-up rewrites it). These are the variants of the steps launched once per
+   level; passes of small 2-D models that are expected to be faster with the
+   wavefields kept on the chip (one launch per pass) still run that way.
+   fwi_autotune_set() pins the per-level steps for its shape; fwi_autotune_reset()
+   forgets all choices.
    3-D grids (opts as for a 3-D gradient: ckpt = FWI_CKPT_SNAPSHOT): the
    compiled ring-depth / CTAs-per-SM variants of the 3-D forward and backward
    steps are timed on the first shot group, keyed by padded shape and group
