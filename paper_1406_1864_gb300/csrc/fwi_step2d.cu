@@ -774,7 +774,7 @@ __global__ void __launch_bounds__(TPB, MINB) k_bwd_step(const __grid_constant__ 
     const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
     const int m = a0.m;
     const bool recon = a0.recon != 0;
-    const bool need_band = recon && m >= 3; // u^{m-2} in the sponge comes from checkpoint m-2 >= 1
+    const bool need_band = !QIN && recon && m >= 3; // u^{m-2} in the sponge comes from checkpoint m-2 >= 1
 
     pdl_trigger();
     if (threadIdx.x == 0) {
@@ -1068,7 +1068,8 @@ __global__ void __launch_bounds__(TPB, MINB) k_bwd_step(const __grid_constant__ 
                     }
                     float pnew[4] = {pn[0].x, pn[0].y, pn[1].x, pn[1].y};
                     float unew[4] = {un[0].x, un[0].y, un[1].x, un[1].y};
-                    if (sg.brow[r] >= 0) {
+                    if (QIN) { // (no rebuild)
+                    } else if (sg.brow[r] >= 0) {
                         unew[0] = bnow[r].x; unew[1] = bnow[r].y; unew[2] = bnow[r].z; unew[3] = bnow[r].w;
                     } else if (sg.any(r)) {
 #pragma unroll
