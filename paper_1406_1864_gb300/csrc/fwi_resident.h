@@ -40,7 +40,7 @@ struct ResArgs {
     float src_scale;
     int ns, nt, nrec;
     int *status;
-    uint2 *xch;            // packets {value, level}: [sets * s][parity][field][ntx * ntz][ne][4]
+    uint2 *xch;            // packets {value, level}: [sets * s][buffer][field][ntx * ntz][ne][4]
     const int *rptr;       // receivers of (tile, shot): [ptr[t * ns + s], ptr[t * ns + s + 1])
     const int2 *rent;      // {local = row * 4 w4 + column, r}
     float *u[2];           // wavefields of even / odd levels, field layout
@@ -58,6 +58,14 @@ struct ResArgs {
     float adj_scale;
     float *acc_grad;       // [nzp][nxp]
 };
+
+// Packet buffer (0 or 1) of level v of a round: the parity of the exchange's number
+// over all rounds, round (nt - 2) + v (levels 1 .. nt - 2 are exchanged in every
+// round of both passes), see fwi_resident2d.cu
+__host__ __device__ inline int res_slot(int round, int nt, int v)
+{
+    return (int)(((unsigned)round * (unsigned)nt + (unsigned)v) & 1u);
+}
 
 // Layout of a pass over ns shots (ok = 0 where one shot does not fit the
 // chip or the streaming steps are expected to be faster)

@@ -9,10 +9,10 @@
 // depends on its neighbours through a 4-cell halo only. Here one cooperative
 // launch runs a whole time loop. A shot's padded grid is cut into tiles, one
 // CTA each; the CTA keeps its tile (and halo) of S shots in shared memory for
-// all levels and goes on to the next S shots when they are done. Per level
-// and shot only the tile's outer 4 rows and columns are exchanged, through
-// the wavefield buffers in L2, and the sponge checkpoint, the traces and the
-// adjoint source touch HBM.
+// all levels and goes on to the next S shots (the next round) when they are done.
+// Per level and shot only the tile's outer 4 rows and columns are exchanged, as
+// packets through L2, and the sponge checkpoint, the traces and the adjoint
+// source touch HBM.
 //
 // Exchange. After a level's compute warps have arrived on the shot's `done`
 // barrier, the export warp sends the tile's outer 4 rows and columns to global
@@ -21,10 +21,19 @@
 // halo in shared memory and arrive on the shot's `full` barrier, which the
 // compute warps wait on. A packet is one access, so neither side needs a fence
 // or a flag: a first version with flags (fence, flag, poll, fence, copy) took
-// about 4 us per exchange. Packets alternate between two buffers by the level's
-// parity: a tile sends level v once it has computed it from the neighbours'
-// level v - 1, which they sent after they had read its level v - 2. While one
-// shot's halo travels, the compute warps advance the other S - 1 shots.
+// about 4 us per exchange. While one shot's halo travels, the compute warps
+// advance the other S - 1 shots.
+//
+// Packets alternate between two buffers. A tile makes its exchanges in one
+// order, k = 1, 2, ... over all rounds, and sends the k-th once it has the
+// (k - 1)-th of its neighbours: within a round because level v is computed from
+// their level v - 1, after a round's end because the round ended with their
+// last one. The neighbours in turn sent their (k - 1)-th after they had read this
+// tile's (k - 2)-th. So the buffer of exchange k - 2 is free, and k & 1 picks the
+// buffer. The level's own parity would not do: a round has nt - 2 exchanges,
+// and with nt odd the next round's level 1, which a tile computes from no packet
+// at all, would land on the last level's packets while a neighbour held up
+// elsewhere may still have to read them.
 //
 // Phases. full[s] of a level completes when the halo has arrived (32 lanes of
 // an import warp), the data warp has the level's amplitudes and adjoint source
@@ -415,7 +424,7 @@ __device__ __forceinline__ void res_init(ResShared &sh, int nw)
 // 0 .. nlev - 1 (forward: the time level, nlev = nt; backward: v = nt - 1 - m,
 // nlev = nt - 1); the first nstep of them are followed by a step. pf, pd:
 // phases of full and done before this round. xb: packets of the CTA's slots,
-// [slot][parity][field][tile][ne][4].
+// [slot][buffer][field][tile][ne][4].
 
 // parity of the buffer that holds level v = 0's current fields: u^0 forward,
 // u^{m-1} with m = nt - 1 backward
@@ -428,7 +437,7 @@ __device__ __forceinline__ int first_parity(int nf, int nt) { return nf == 2 ? (
 template <int NF>
 __device__ __noinline__ void service_export(const ResArgs &a, float *sm, const Xch *xt, const int2 *bl, uint2 *xb,
                                             ResShared *sh, int tile, int b0, int shot0, int nsh, int nlev, int nstep,
-                                            uint32_t pd, uint32_t tag0)
+                                            uint32_t pd, uint32_t tag0, int round)
 {
     const int lane = threadIdx.x & 31, ne = a.t.ne, ntiles = a.t.ntx * a.t.ntz, fs = a.t.fs, nt = a.nt;
     const long long blk = (long long)ntiles * ne * 4;
@@ -475,7 +484,7 @@ __device__ __noinline__ void service_export(const ResArgs &a, float *sm, const X
 #pragma unroll
                 for (int f = 0; f < NF; ++f) {
                     const float *fl = sm + (2 * NF * s + 2 * f + b) * fs;
-                    uint2 *out = xb + ((s * 2 + (v & 1)) * NF + f) * blk + (long long)tile * ne * 4;
+                    uint2 *out = xb + ((s * 2 + res_slot(round, nt, v)) * NF + f) * blk + (long long)tile * ne * 4;
 #pragma unroll 2
                     for (int e = lane; e < ne; e += 32) {
                         if (xt[e].src < 0) continue;
@@ -493,7 +502,8 @@ __device__ __noinline__ void service_export(const ResArgs &a, float *sm, const X
 // Import warp h: the halos of shots h, h + RES_IMPORT, ...
 template <int NF>
 __device__ __noinline__ void service_import(float *sm, const Xch *xt, const uint2 *xb, ResShared *sh, int ne, int ntiles,
-                                            int fs, int b0, int nsh, int nlev, int nstep, uint32_t pf, uint32_t tag0, int h)
+                                            int fs, int b0, int nsh, int nlev, int nstep, uint32_t pf, uint32_t tag0,
+                                            int round, int nt, int h)
 {
     const int lane = threadIdx.x & 31;
     for (int s = h; s < nsh; s += RES_IMPORT) mbar_arrive(smem_u32(&sh->bars.full[s])); // level 0: in place
@@ -509,7 +519,7 @@ __device__ __noinline__ void service_import(float *sm, const Xch *xt, const uint
 #pragma unroll
                 for (int f = 0; f < NF; ++f) {
                     float *fl = sm + (2 * NF * s + 2 * f + b) * fs;
-                    const uint2 *in = xb + ((s * 2 + (v & 1)) * NF + f) * blk;
+                    const uint2 *in = xb + ((s * 2 + res_slot(round, nt, v)) * NF + f) * blk;
                     constexpr int B = 4; // float4s in flight per lane
                     for (int e0 = lane; e0 < ne; e0 += 32 * B) {
                         uint64_t q[B][4];
@@ -864,9 +874,9 @@ __global__ void __launch_bounds__(32 * (NW + RES_SVC), 1) k_fwd_resident(const _
             const int ntiles = t.ntx * t.ntz;
             uint2 *xb = a.xch + (long long)c.set * t.s * 2 * ntiles * t.ne * 4;
             if (wid == NW)
-                service_export<1>(a, sm, xt, bl, xb, &sh, c.tile, 0, first + base, nsh, nt, nt - 1, pd, pf);
+                service_export<1>(a, sm, xt, bl, xb, &sh, c.tile, 0, first + base, nsh, nt, nt - 1, pd, pf, round);
             else if (wid <= NW + RES_IMPORT)
-                service_import<1>(sm, xt, xb, &sh, t.ne, ntiles, fs, 0, nsh, nt, nt - 1, pf, pf, wid - NW - 1);
+                service_import<1>(sm, xt, xb, &sh, t.ne, ntiles, fs, 0, nsh, nt, nt - 1, pf, pf, round, nt, wid - NW - 1);
             else
                 service_traces(a, sm, list, bl, &sh, first + base, nsh, pd);
         }
@@ -1135,9 +1145,9 @@ __global__ void __launch_bounds__(32 * (NW + RES_SVC), 1) k_bwd_resident(const _
             const int ntiles = t.ntx * t.ntz, b0 = first_parity(2, nt);
             uint2 *xb = a.xch + (long long)c.set * t.s * 4 * ntiles * t.ne * 4;
             if (wid == NW)
-                service_export<2>(a, sm, xt, bl, xb, &sh, c.tile, b0, first + base, nsh, nt - 1, nt - 1, p0, p0);
+                service_export<2>(a, sm, xt, bl, xb, &sh, c.tile, b0, first + base, nsh, nt - 1, nt - 1, p0, p0, round);
             else if (wid <= NW + RES_IMPORT)
-                service_import<2>(sm, xt, xb, &sh, t.ne, ntiles, fs, b0, nsh, nt - 1, nt - 1, p0, p0, wid - NW - 1);
+                service_import<2>(sm, xt, xb, &sh, t.ne, ntiles, fs, b0, nsh, nt - 1, nt - 1, p0, p0, round, nt, wid - NW - 1);
             else
                 service_adjoint(a, inj, &sh, first + base, nsh, p0);
         }
