@@ -2719,6 +2719,7 @@ fwi_status fwi_workspace_preferred_bytes(int nmodels, const fwi_grid *grids, con
                                          const fwi_options *opts, int op, size_t *bytes)
 {
     if (!bytes) return fail(FWI_ERR_INVALID_ARG, "bytes is NULL");
+    if (nmodels < 1) return fail(FWI_ERR_INVALID_ARG, "nmodels=%d outside 1..%d", nmodels, FWI_BATCH_MAX);
     const bool two = grids && grids[0].ndim == 2;
     if (op == FWI_OP_GRADIENT && two && opts) {
         std::vector<Plan> pl;
