@@ -177,7 +177,10 @@ fwi_status fwi_workspace_bytes(const fwi_grid *grid, const fwi_geometry *geom,
    the offset Hessian keep the levels of their forward pass (at most 4 GiB per
    model) and sum over them at the end. With less, down to the sizes of those
    functions, the sums are taken after every level; the results agree to FP32
-   rounding. grids, geoms: HOST arrays [nmodels]. */
+   rounding. The levels count where the call will keep them: not for shapes
+   pinned with fwi_autotune_set(), a batch whose forward pass runs batched, or
+   (where the geometry's arrays are given) receivers too dense for such a pass.
+   grids, geoms: HOST arrays [nmodels]. */
 fwi_status fwi_workspace_preferred_bytes(int nmodels, const fwi_grid *grids, const fwi_geometry *geoms,
                                          const fwi_options *opts, int op, size_t *bytes);
 

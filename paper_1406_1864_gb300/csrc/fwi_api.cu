@@ -312,7 +312,6 @@ fwi_status make_plan(const fwi_grid *g, const fwi_geometry *ge, const fwi_option
     if (allow_resident && (!pl.snap || o->snap_prec == FWI_SNAP_F32) && !(born && !need_bwd) && op != FWI_OP_GN_HVP)
         pl.rf = choose_resident(L, pl.ns, res_forward_kind(o, op), pl.with_offh ? hist_bytes(L, pl.ns, pl.nt) : 0);
     const StepKind fkind = pl.with_offh ? STEP_FWD_OFFH : STEP_FWD;
-    const size_t hist = pl.rf.ok && pl.with_offh ? hist_bytes(L, pl.ns, pl.nt) : 0;
     if (allow_resident && need_bwd && !pl.snap) pl.rb = choose_resident(L, pl.ns, RES_BWD);
     // (the workspace does not depend on pinned steps or the receivers' places,
     // and extended migration holds the state of a plain adjoint pass)
@@ -321,6 +320,7 @@ fwi_status make_plan(const fwi_grid *g, const fwi_geometry *ge, const fwi_option
     if (pl.ext) pl.rb = ResTile{};
     if (pl.rf.ok && (res_pinned(fkind, L, pl.ns) || (coords && !receivers_fit(L, ge, pl.rf, false)))) pl.rf = ResTile{};
     if (pl.rb.ok && (res_pinned(STEP_BWD, L, pl.ns) || (coords && !receivers_fit(L, ge, pl.rb, true)))) pl.rb = ResTile{};
+    const size_t hist = pl.rf.ok && pl.with_offh ? hist_bytes(L, pl.ns, pl.nt) : 0;
     const size_t fbytes = (size_t)L.fstride * sizeof(float);
     const size_t nphys = (size_t)L.nz * L.nx;
     take(pl.c2, fbytes);
@@ -1893,12 +1893,6 @@ fwi_status make_batch(int nm, const fwi_grid *grids, const fwi_geometry *geoms, 
         base[k] = total;
         total = align_up(total + pl[k].total);
     }
-    // the kept levels of resident forward passes follow the models' slices
-    preferred = total;
-    for (int k = 0; k < nm; ++k) {
-        pl[k].hist.off = preferred - base[k];
-        preferred = align_up(preferred + pl[k].hist.bytes);
-    }
     // a launch runs one kernel for all models: the tile variants and chunks
     // of the model with the most work (padded points x shots); the workspace
     // does not depend on the tiling
@@ -1919,6 +1913,13 @@ fwi_status make_batch(int nm, const fwi_grid *grids, const fwi_geometry *geoms, 
         }
         if (all && us < streaming_us(pts, b ? RES_BWD : RES_FWD_U2)) continue;
         for (int k = 0; k < nm; ++k) (b ? pl[k].rb : pl[k].rf) = ResTile{};
+    }
+    // the kept levels of resident forward passes follow the models' slices
+    preferred = total;
+    for (int k = 0; k < nm; ++k) {
+        if (!pl[k].rf.ok) pl[k].hist.bytes = 0;
+        pl[k].hist.off = preferred - base[k];
+        preferred = align_up(preferred + pl[k].hist.bytes);
     }
     for (int k = 0; k < nm; ++k) {
         if (k == kmax) continue;
@@ -2721,11 +2722,15 @@ fwi_status fwi_workspace_preferred_bytes(int nmodels, const fwi_grid *grids, con
     if (!bytes) return fail(FWI_ERR_INVALID_ARG, "bytes is NULL");
     if (nmodels < 1) return fail(FWI_ERR_INVALID_ARG, "nmodels=%d outside 1..%d", nmodels, FWI_BATCH_MAX);
     const bool two = grids && grids[0].ndim == 2;
+    // (whether the receivers suit a resident pass, where their places are given)
+    bool coords = two && geoms && opts && opts->hmax >= 0 && nmodels <= FWI_BATCH_MAX;
+    for (int k = 0; coords && k < nmodels; ++k)
+        coords = geoms[k].src && geoms[k].wavelet && (geoms[k].rec || geoms[k].nrec == 0);
     if (op == FWI_OP_GRADIENT && two && opts) {
         std::vector<Plan> pl;
         std::vector<size_t> base;
         size_t total = 0;
-        fwi_status s = make_batch(nmodels, grids, geoms, opts, false, pl, base, total, *bytes);
+        fwi_status s = make_batch(nmodels, grids, geoms, opts, coords, pl, base, total, *bytes);
         if (s == FWI_OK) t_err.clear();
         return s;
     }
@@ -2733,7 +2738,7 @@ fwi_status fwi_workspace_preferred_bytes(int nmodels, const fwi_grid *grids, con
     fwi_status s = fwi_workspace_bytes(grids, geoms, opts, op, bytes);
     if (s != FWI_OK || op != FWI_OP_OFFSET_HESSIAN || !two) return s;
     Plan pl;
-    if ((s = make_plan(grids, geoms, opts, op, false, pl)) != FWI_OK) return s;
+    if ((s = make_plan(grids, geoms, opts, op, coords, pl)) != FWI_OK) return s;
     *bytes = pl.hist.off + pl.hist.bytes;
     t_err.clear();
     return FWI_OK;
