@@ -152,6 +152,7 @@ class Workspace:
     def __init__(self, device=None):
         self.device = device or torch.device("cuda", torch.cuda.current_device())
         self.buf = None
+        self.refused = None  # smallest size that could not be allocated
 
     def get(self, nbytes: int) -> torch.Tensor:
         if self.buf is None or self.buf.numel() < nbytes:
@@ -160,10 +161,21 @@ class Workspace:
         return self.buf
 
 
-def _ws(ws, nbytes):
+def _ws(ws, nbytes, least=None):
+    """Buffer of a call. least: function of the size the call needs where nbytes
+    is that of its fastest path, taken when there is no memory for nbytes (and by
+    later calls on the same Workspace, which do not try again)."""
     if ws is None:
         ws = Workspace()
-    buf = ws.get(nbytes) if isinstance(ws, Workspace) else ws
+    if not isinstance(ws, Workspace):
+        return ws, ws.numel()
+    if least is not None and (ws.refused is None or nbytes < ws.refused):
+        try:
+            buf = ws.get(nbytes)
+            return buf, buf.numel()
+        except torch.cuda.OutOfMemoryError:
+            ws.refused = nbytes
+    buf = ws.get(nbytes if least is None else least())
     return buf, buf.numel()
 
 
@@ -219,7 +231,8 @@ def adjoint_gradient(grid: Grid, geom: Geometry, v: torch.Tensor, d_obs: torch.T
     if want_offh:
         res["offh"] = o.get("offh", torch.empty((opts.hmax + 1,) + grid.shape, dtype=torch.float32,
                                                 device=dev))
-    buf, nb = _ws(ws, preferred_workspace_bytes([grid], [geom], opts, "gradient"))
+    buf, nb = _ws(ws, preferred_workspace_bytes([grid], [geom], opts, "gradient"),
+                  lambda: workspace_bytes(grid, geom, opts, "gradient"))
     g, ge, oc = grid.c(), geom.c(), opts.c()
     L.check(L.load().fwi_adjoint_gradient(
         ctypes.byref(g), ctypes.byref(ge), ctypes.byref(oc), _ptr(v), _ptr(d_obs), _ptr(res["grad"]),
@@ -280,7 +293,8 @@ def batch_gradient(grids, geoms, vs, d_obs, opts: Options | None = None, *, want
     Returns one dict per model, as adjoint_gradient."""
     opts = opts or Options()
     res, c = _batch_args(grids, geoms, vs, d_obs, opts, want_pre, want_illum, want_offh)
-    buf, nb = _ws(ws, preferred_workspace_bytes(grids, geoms, opts, "gradient"))
+    buf, nb = _ws(ws, preferred_workspace_bytes(grids, geoms, opts, "gradient"),
+                  lambda: batch_workspace_bytes(grids, geoms, opts))
     L.check(L.load().fwi_batch_gradient(len(grids), c["g"], c["ge"], ctypes.byref(c["o"]), c["v"], c["d"],
                                         c["grad"], c["pre"], _ptr(c["misfit"]), c["ill"], c["off"], _ptr(buf),
                                         nb, _stream(stream)), "fwi_batch_gradient")
@@ -300,7 +314,8 @@ class GradientGraph:
         self.inputs = (list(vs), list(d_obs))
         self.results, c = _batch_args(grids, geoms, vs, d_obs, opts, want_pre, want_illum, want_offh)
         self._c = c  # keep the ctypes arrays alive with the graph
-        self.buf, nb = _ws(ws, preferred_workspace_bytes(grids, geoms, opts, "gradient"))
+        self.buf, nb = _ws(ws, preferred_workspace_bytes(grids, geoms, opts, "gradient"),
+                           lambda: batch_workspace_bytes(grids, geoms, opts))
         self.stream = torch.cuda.Stream(device=vs[0].device)
         self.stream.wait_stream(torch.cuda.current_stream())
         h = ctypes.c_void_p(0)
@@ -447,7 +462,8 @@ def offset_hessian_diag(grid: Grid, geom: Geometry, v: torch.Tensor, opts: Optio
     offset-Hessian diagonal, offsets along x."""
     _dev(v, "v", grid.shape)
     out = torch.empty((opts.hmax + 1,) + grid.shape, dtype=torch.float32, device=v.device)
-    buf, nb = _ws(ws, preferred_workspace_bytes([grid], [geom], opts, "offset_hessian"))
+    buf, nb = _ws(ws, preferred_workspace_bytes([grid], [geom], opts, "offset_hessian"),
+                  lambda: workspace_bytes(grid, geom, opts, "offset_hessian"))
     g, ge, oc = grid.c(), geom.c(), opts.c()
     L.check(L.load().fwi_offset_hessian_diag(ctypes.byref(g), ctypes.byref(ge), ctypes.byref(oc),
                                              _ptr(v), _ptr(out), _ptr(buf), nb, _stream(stream)),

@@ -5,6 +5,7 @@ import subprocess
 import sys
 
 import numpy as np
+import pytest
 
 ROOT = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
 
@@ -80,3 +81,64 @@ def test_levels_count_only_where_the_call_keeps_them():
         assert more == need
     finally:
         fwi.autotune_reset()
+
+
+def _tight(limit, device):
+    """a Workspace on a device without room for more than limit bytes"""
+    import torch
+    from paper_1406_1864_gb300 import fwi
+
+    class Tight(fwi.Workspace):
+        tries = 0
+
+        def get(self, nbytes):
+            if nbytes > limit:
+                Tight.tries += 1
+                raise torch.cuda.OutOfMemoryError("no room")
+            return super().get(nbytes)
+
+    return Tight(torch.device(device))
+
+
+def test_a_refused_allocation_falls_back_to_the_size_the_call_needs():
+    import torch
+    from paper_1406_1864_gb300 import fwi
+    ws = _tight(1000, "cpu")
+    for _ in range(2):  # (the second call does not try again)
+        buf, n = fwi._ws(ws, 5000, lambda: 800)
+        assert n >= 800 and buf is ws.buf and type(ws).tries == 1
+    buf, n = fwi._ws(ws, 900, lambda: 300)
+    assert n >= 900
+    with pytest.raises(torch.cuda.OutOfMemoryError):
+        fwi._ws(ws, 2000)
+    with pytest.raises(torch.cuda.OutOfMemoryError):
+        fwi._ws(_tight(1000, "cpu"), 5000, lambda: 4000)
+
+
+@pytest.mark.gpu
+def test_calls_without_room_for_their_levels_run():
+    """Every call that asks for the preferred size runs with the required one:
+    the sums after each level, the same to FP32 rounding (1e-5, as between a
+    workspace with and without room for the levels)."""
+    import torch
+    from paper_1406_1864_gb300 import fwi, workloads as W
+    p = W.dipping(nz=37, nx=83, nt=60, ns=3, nrec=83, sponge=7)
+    grid, geom = fwi.from_problem(p)
+    v = torch.as_tensor(p.v_init, device="cuda")
+    d = fwi.forward(grid, geom, torch.as_tensor(p.v_true, device="cuda"))
+    opts = fwi.Options(hmax=10, precond="offset")
+    calls = {"gradient": lambda ws: fwi.adjoint_gradient(grid, geom, v, d, opts, ws=ws),
+             "batch": lambda ws: fwi.batch_gradient([grid] * 2, [geom] * 2, [v] * 2, [d] * 2, opts, ws=ws)[1],
+             "graph": lambda ws: fwi.GradientGraph([grid], [geom], [v], [d], opts, ws=ws).run()[0],
+             "offset_hessian": lambda ws: {"offh": fwi.offset_hessian_diag(grid, geom, v, opts, ws=ws)}}
+    need = {"gradient": fwi.workspace_bytes(grid, geom, opts, "gradient"),
+            "batch": fwi.batch_workspace_bytes([grid] * 2, [geom] * 2, opts),
+            "graph": fwi.batch_workspace_bytes([grid], [geom], opts),
+            "offset_hessian": fwi.workspace_bytes(grid, geom, opts, "offset_hessian")}
+    for name, call in calls.items():
+        full, ws = call(None), _tight(need[name], "cuda")
+        res = call(ws)
+        assert type(ws).tries == 1, name
+        for k in ("offh", "grad"):
+            if k in full:
+                assert float((res[k] - full[k]).double().norm()) <= 1e-5 * float(full[k].double().norm()), (name, k)
