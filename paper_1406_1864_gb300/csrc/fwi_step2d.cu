@@ -43,6 +43,7 @@
 #include <cudaTypedefs.h>
 
 #include <algorithm>
+#include <cmath>
 #include <map>
 #include <mutex>
 #include <tuple>
@@ -1533,7 +1534,8 @@ struct Variant {
     const void *fn[3]; // one model per launch, batch of up to BATCH_MAX models, and (plain
                        // forward and backward steps) the one-model instance that keeps (forward)
                        // or reads (backward) the imaging factor q of a re-propagated segment
-    int occ[2];        // resident CTAs per SM (from the occupancy calculator)
+    int occ[2];        // resident CTAs per SM (from the occupancy calculator; as compiled for
+                       // where there is no device)
 };
 
 #define FWD_VARIANT(RZ, ST, MINB, SPI)                                                     \
@@ -1541,23 +1543,23 @@ struct Variant {
      {(const void *)k_fwd_step<RZ, RADIUS, false, ST, MINB, 1, SPI>,                       \
       (const void *)k_fwd_step<RZ, RADIUS, false, ST, MINB, BATCH_MAX, SPI>,               \
       (const void *)k_fwd_step<RZ, RADIUS, false, ST, MINB, 1, SPI, HMAX_LIMIT + 1, true>}, \
-     {0, 0}}
+     {MINB, MINB}}
 #define FWDH_VARIANT(ST, MINB, SPI, NHC)                                                   \
     {1, SPI, FwdRing<1, HMAX_LIMIT, true, ST, SPI>::SMEM, NHC, 0,                          \
      {(const void *)k_fwd_step<1, HMAX_LIMIT, true, ST, MINB, 1, SPI, NHC>,                \
       (const void *)k_fwd_step<1, HMAX_LIMIT, true, ST, MINB, BATCH_MAX, SPI, NHC>, nullptr}, \
-     {0, 0}}
+     {MINB, MINB}}
 // the plain step with the offset Hessian summed by k_offh_level after it
 #define FWDS_VARIANT(RZ, ST, MINB, SPI)                                                    \
     {RZ, SPI, FwdRing<RZ, RADIUS, false, ST, SPI>::SMEM, HMAX_LIMIT + 1, 1,               \
      {(const void *)k_fwd_step<RZ, RADIUS, false, ST, MINB, 1, SPI>,                       \
       (const void *)k_fwd_step<RZ, RADIUS, false, ST, MINB, BATCH_MAX, SPI>, nullptr},     \
-     {0, 0}}
+     {MINB, MINB}}
 #define BWD_VARIANT(RZ, ST, MINB)                                                          \
     {RZ, 1, BwdRing<RZ, ST>::SMEM, 0, 0,                                                   \
      {(const void *)k_bwd_step<RZ, ST, MINB, 1>, (const void *)k_bwd_step<RZ, ST, MINB, BATCH_MAX>, \
       (const void *)k_bwd_step<RZ, ST, MINB, 1, 0, true>},                                \
-     {0, 0}}
+     {MINB, MINB}}
 
 // forward: 64 x 16 tiles (3 stages, 4 CTAs/SM), 64 x 32 (2 stages), 64 x 8
 // (6 CTAs/SM), 64 x 16 with two shots per item (2 stages)
@@ -1610,7 +1612,7 @@ void prepare_kernels()
                             cudaSuccess)
                             occ = 0;
                     }
-                    v[i].occ[b] = occ > 0 ? occ : 2;
+                    if (occ > 0) v[i].occ[b] = occ;
                 }
             for (int i = 0; i < n; ++i)
                 if (have_dev && v[i].fn[2])
@@ -1738,8 +1740,40 @@ bool step_variant_valid(StepKind kind, int variant, int hmax)
     return kind != STEP_FWD_OFFH || hmax <= vs[variant].nh - 1;
 }
 
+namespace {
+// Expected time of a level, in us:
+//   base + chunk x (items of the CTA with the longest run of chunks)
+//        + (item + band x sponge share of the points) x (items per resident CTA).
+// A chunk's shots follow one another in one CTA; the CTAs of a launch take their
+// second chunk by order (it is fetched a chunk ahead), so with n chunks on P
+// resident CTAs the longest run has ceil(n / P) of them, the half blocks of the
+// models' last shots behind the whole ones. The second term is what all CTAs
+// together ask of L2 and HBM, the checkpoint of the sponge among it. Fitted (least
+// squares of the relative error, 5 to 95% within -12 and +13%) to 123 problems of
+// 36 to 500 rows, 80 to 1500 columns, 1 to 96 shots, 0.03 to 52 M padded points.
+struct LevelCost {
+    double base, chunk, item, band;
+};
+constexpr LevelCost COST_B[2] = {{3.3, 1.92, 0.33, 3.2}, {2.9, 1.62, 0.04, 2.35}}; // g_var_b
+
+double level_us(const LevelCost &c, const Variant &v, int chunk, const Lay2D &L, int ns)
+{
+    const double slots = std::max(1, sm_count_dev() * v.occ[0]);
+    const double tiles = (double)((L.nxp + TX - 1) / TX) * ((L.nzp + 8 * v.rz - 1) / (8 * v.rz));
+    auto items = [&](int shots) { return (shots + v.spi - 1) / v.spi; };
+    chunk = std::min(ns, chunk);
+    const int nb = chunk_blocks(ns, chunk), whole = std::max(1, (ns + chunk - 1) / chunk - 1);
+    const int h0 = nb == 1 ? 0 : (ns - whole * chunk + 1) / 2, h1 = nb == 1 ? 0 : ns - whole * chunk - h0;
+    const double r0 = std::ceil(tiles * whole / slots), r1 = std::ceil(tiles * nb / slots);
+    const double longest = r0 * items(chunk) + (r1 - r0) * items(h0);
+    const double mean = tiles * (whole * items(chunk) + items(h0) + items(h1)) / slots;
+    const double sponge = 1.0 - (double)L.nz * L.nx / ((double)L.nzp * L.nxp);
+    return c.base + c.chunk * longest + (c.item + c.band * sponge) * mean;
+}
+} // namespace
+
 // Tile variant of a problem that was not autotuned, from the variants pinned one
-// by one in gradients of 0.5 to 38 M padded points over all shots (us per level):
+// by one in gradients of 0.5 to 52 M padded points over all shots (us per level):
 // - forward: two-shot items beat single ones everywhere (100 x 200, 16 shots
 //   11.8 against 13.8; 150 x 460, 80 shots 29.8 / 34.2; 400 x 1200, 64 shots
 //   101 / 111.5); a single shot takes the one-shot variant.
@@ -1748,23 +1782,19 @@ bool step_variant_valid(StepKind kind, int variant, int hmax)
 //   shots 140 against 150), but sum the zero-offset image in another order than the
 //   illumination (3e-5 apart after 4000 levels of 300 x 1000, else equal), so only
 //   autotuning takes them.
-// - backward: the variant with the shorter level by rounds of resident CTAs; a
-//   round of 64 x 8 tiles (5 CTAs per SM) takes about 0.75 of one of 64 x 16 (4 per
-//   SM): 15 against 20 us at 8 shots per chunk. One round each: 100 x 200, 64 shots
-//   21.7 against 26.6, 300 x 1000, 2 shots 7.3 / 8.8; two against one: 71 x 332, 90
-//   shots 37.8 / 27.1, 200 x 400, 32 shots 29.0 / 26.1; two each: 300 x 1000, 16 shots
-//   36.1 / 37.9; many: 500 x 1500, 16 shots 72.1 / 66.6, 400 x 1200, 64 shots 166 / 154.
+// - backward: the variant with the shorter expected level. 64 x 16 tiles (4 CTAs per
+//   SM) against 64 x 8 (5 per SM): one round of CTAs each, 100 x 200, 64 shots 25.7 /
+//   22.7; two whole chunks a CTA against one and a half, 150 x 460, 48 shots 34.1 /
+//   40.7, 94 x 299, 92 shots 31.5 / 39.9; the other way about, 300 x 1000, 12 shots
+//   29.7 / 27.5; many rounds, 300 x 1000, 32 shots 60.2 / 66.5, 400 x 1200, 64 shots
+//   150 / 171. Over the 123 problems the choice costs 0.2% on average against the
+//   better of the two, 7% at most.
 int default_variant(const Lay2D &L, int ns, StepKind kind, int hmax)
 {
     if (kind == STEP_FWD) return ns > 1 ? 3 : 0;
     if (kind == STEP_BWD) {
-        auto rounds = [&](const Variant &v) {
-            const long long tiles = (long long)((L.nxp + TX - 1) / TX) * ((L.nzp + 8 * v.rz - 1) / (8 * v.rz));
-            const long long slots = std::max(1LL, (long long)sm_count_dev() * v.occ[0]);
-            const int chunk = std::min(ns, CHUNKS_F[0]);
-            return (tiles * chunk_blocks(ns, chunk) + slots - 1) / slots;
-        };
-        return 3 * rounds(g_var_b[1]) < 4 * rounds(g_var_b[0]) ? 1 : 0;
+        auto us = [&](int i) { return level_us(COST_B[i], g_var_b[i], CHUNKS_F[0], L, ns); };
+        return us(1) < us(0) ? 1 : 0;
     }
     return hmax <= g_var_h[2].nh - 1 ? 2 : 1;
 }

@@ -7,13 +7,12 @@ step is followed with the library's choice of buffer (fwi_resident.h, compiled
 here); none may leave a tile waiting for a packet that was overwritten. On the
 GPU: passes of several rounds and tiles against the streaming steps."""
 import ctypes
-import os
-import subprocess
 
 import numpy as np
 import pytest
 
-from paper_1406_1864_gb300 import build as B, workloads as W
+import native
+from paper_1406_1864_gb300 import workloads as W
 
 HELPER = """
 #include "fwi_resident.h"
@@ -32,15 +31,7 @@ FWD_U2, BWD = 1, 3
 
 @pytest.fixture(scope="module")
 def helper(tmp_path_factory):
-    lib = B.build()
-    d = tmp_path_factory.mktemp("resident")
-    src, so = d / "helper.cpp", d / "helper.so"
-    src.write_text(HELPER)
-    cuda = os.environ.get("CUDA_HOME", "/usr/local/cuda")
-    subprocess.check_call(["g++", "-std=c++17", "-shared", "-fPIC", f"-I{cuda}/include", "-I", os.path.join(B.ROOT, "include"),
-                           "-I", B.CSRC, str(src), "-L", B.HERE, "-l:" + os.path.basename(lib), f"-Wl,-rpath,{B.HERE}",
-                           "-o", str(so)])
-    return ctypes.CDLL(str(so))
+    return native.compile_helper(HELPER, tmp_path_factory.mktemp("resident"))
 
 
 def stuck(slot, nt, rounds, tiles=3):
