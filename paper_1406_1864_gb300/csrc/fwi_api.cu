@@ -220,30 +220,34 @@ bool receivers_fit(const Lay2D &L, const fwi_geometry *ge, const ResTile &t, boo
     return true;
 }
 
-// Level of the streaming steps in us, fitted to the measured ones from 0.1 M to
-// 17 M padded points: forward 7.1, 14.9, 15.7, 23.4 and 29.8 us at 0.13, 2.2, 3.4,
-// 5.7 and 7.6 M; backward 9.2, 21.7, 26.8, 36.1, 50.1 and 87 us at 0.13, 2.2, 3.4,
-// 5.7, 7.6 and 17 M.
-double streaming_us(double pts, ResKind kind)
-{
-    return kind == RES_BWD ? std::min(8.0 + 9e-6 * pts, 11.0 + 4.8e-6 * pts)
-                           : std::min(6.0 + 4.0e-6 * pts, 9.0 + 2.6e-6 * pts);
-}
-
 // The levels that a resident forward pass keeps for the offset-Hessian sums
 size_t hist_bytes(const Lay2D &L, int ns, int nt) { return (size_t)(nt - 1) * ns * L.fstride * sizeof(float); }
 constexpr size_t HIST_MAX = size_t(4) << 30;
 
-// The resident time loop where it is expected to be faster; hist > 0: with the
-// offset Hessian, whose sums take about the same time on kept levels (for the
-// writing of which 0.7 us per M points is allowed) as after each streaming step
-// (which adds a launch to each).
-ResTile choose_resident(const Lay2D &L, int ns, ResKind kind, size_t hist = 0)
+// The resident time loop where it is expected to be faster than the streaming steps
+// (step_level_us). hist > 0: with the offset Hessian, summed in the streaming step;
+// the levels that a resident pass keeps instead cost 1.7 us per M points to write
+// and sum. Over 123 problems of 0.03 to 52 M padded points the choice costs, on
+// average against the better loop, 0.1% (plain), 0.7% (checkpoint), 0.2% (checkpoint and
+// illumination), 0.3% (illumination), 0.2% (backward) and 0.4% (offset Hessian); over 110
+// others 0.0, 0.4, 0.1, 0.6, 0.7 and 0.2%. Where the two are near each other a single
+// problem costs up to 24%. us per level, streaming / resident, on both sides:
+//   forward    300 x 1000, 24 shots 28.2 / 25.1, 32 shots 36.6 / 37.2, 96 shots 91.4 /
+//              100.1; 400 x 1200, 4 shots 8.1 / 6.7, 16 shots 26.3 / 28.6, 32 shots 49.3 /
+//              56.5; 150 x 460, 80 shots 27.8 / 19.8; 250 x 700, 48 shots 34.0 / 37.0
+//   checkpoint and illumination
+//              300 x 1000, 12 shots 18.9 / 15.8, 24 shots 31.9 / 34.8; 400 x 1200, 4 shots
+//              8.8 / 9.2, 16 shots 29.5 / 40.1; 150 x 460, 80 shots 32.8 / 31.1
+//   backward   100 x 200, 64 shots 22.4 / 18.1, 96 shots 26.7 / 27.2; 400 x 1200, 2 shots
+//              8.4 / 9.2; 150 x 460, 12 shots 19.4 / 12.1, 24 shots 23.9 / 24.1
+ResTile choose_resident(const Lay2D &L, int ns, ResKind kind, bool band, size_t hist = 0)
 {
-    const ResTile t = res_plan(L, ns, kind);
-    const double pts = (double)L.nzp * L.nxp * ns;
-    const double more = hist > 0 ? 0.7e-6 * pts - 4.0 : 0.0;
-    return t.ok && hist <= HIST_MAX && t.us + more < streaming_us(pts, kind) ? t : ResTile{};
+    ResTile t = res_plan(L, ns, kind);
+    if (!t.ok || hist > HIST_MAX) return ResTile{};
+    const Lay2D *l = &L;
+    const StepKind steps = kind == RES_BWD ? STEP_BWD : (hist > 0 ? STEP_FWD_OFFH : STEP_FWD);
+    t.us = (float)(res_level_us(L, t, kind, band) + (hist > 0 ? 1.7e-6 * L.nzp * L.nxp * ns : 0.0));
+    return t.us < step_level_us(1, &l, &ns, steps, band) ? t : ResTile{};
 }
 
 ResKind res_forward_kind(const fwi_options *o, int op)
@@ -310,9 +314,10 @@ fwi_status make_plan(const fwi_grid *g, const fwi_geometry *ge, const fwi_option
                    : (born ? make_tiling(L, pl.ns, STEP_BWD, 0) : make_tiling(L, pl.ns, STEP_BWD));
     // (16-bit snapshots are scaled by the maxima of a whole field: streaming)
     if (allow_resident && (!pl.snap || o->snap_prec == FWI_SNAP_F32) && !(born && !need_bwd) && op != FWI_OP_GN_HVP)
-        pl.rf = choose_resident(L, pl.ns, res_forward_kind(o, op), pl.with_offh ? hist_bytes(L, pl.ns, pl.nt) : 0);
+        pl.rf = choose_resident(L, pl.ns, res_forward_kind(o, op), need_bwd && !pl.snap,
+                                pl.with_offh ? hist_bytes(L, pl.ns, pl.nt) : 0);
     const StepKind fkind = pl.with_offh ? STEP_FWD_OFFH : STEP_FWD;
-    if (allow_resident && need_bwd && !pl.snap) pl.rb = choose_resident(L, pl.ns, RES_BWD);
+    if (allow_resident && need_bwd && !pl.snap) pl.rb = choose_resident(L, pl.ns, RES_BWD, true);
     // (the workspace does not depend on pinned steps or the receivers' places,
     // and extended migration holds the state of a plain adjoint pass)
     const size_t xch = (size_t)std::max(pl.rf.xch, pl.rb.xch);
@@ -1903,15 +1908,19 @@ fwi_status make_batch(int nm, const fwi_grid *grids, const fwi_geometry *geoms, 
     // a pass of the batch is resident (one launch per model) where that is so
     // for every model and expected to be faster than the batched steps
     for (int b = 0; b < 2 && nm > 1; ++b) {
-        double pts = 0, us = 0;
+        double us = 0;
         bool all = true;
+        std::vector<const Lay2D *> L(nm);
+        std::vector<int> ns(nm);
         for (int k = 0; k < nm; ++k) {
             const ResTile &t = b ? pl[k].rb : pl[k].rf;
             all = all && t.ok;
             us += t.us;
-            pts += (double)pl[k].L.nzp * pl[k].L.nxp * pl[k].ns;
+            L[k] = &pl[k].L;
+            ns[k] = pl[k].ns;
         }
-        if (all && us < streaming_us(pts, b ? RES_BWD : RES_FWD_U2)) continue;
+        const StepKind steps = b ? STEP_BWD : (pl[0].with_offh ? STEP_FWD_OFFH : STEP_FWD);
+        if (all && us < step_level_us(nm, L.data(), ns.data(), steps, true)) continue;
         for (int k = 0; k < nm; ++k) (b ? pl[k].rb : pl[k].rf) = ResTile{};
     }
     // the kept levels of resident forward passes follow the models' slices

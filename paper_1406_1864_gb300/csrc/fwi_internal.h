@@ -40,6 +40,9 @@ cudaError_t launch_precond_n(long long nphys, const float *grad, const float *sc
 // (hmax: the offset Hessian's largest offset, for the variants of
 // STEP_FWD_OFFH, which cover hmax up to a compiled count)
 Tiling make_tiling(const Lay2D &L, int ns, StepKind kind, int variant = -1, int chunk = 0, int hmax = HMAX_LIMIT);
+// expected time (us) of a level of nm models with the default tiles; band: the
+// steps keep or read the sponge checkpoint
+double step_level_us(int nm, const Lay2D *const *L, const int *ns, StepKind kind, bool band);
 bool step_variant_valid(StepKind kind, int variant, int hmax);
 // box sizes (x, y) of the halo and point tiles of a step kernel
 void step_boxes(StepKind kind, const Tiling &t, int &hx, int &hy, int &px, int &py);

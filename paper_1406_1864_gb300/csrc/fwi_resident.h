@@ -28,7 +28,7 @@ struct ResTile {
     int ne;            // float4s of a tile's edge strips
     int smem;          // dynamic shared memory
     long long xch;     // bytes of the exchange packets
-    float us;          // estimated time of one level of all shots, in us
+    float us;          // expected time of one level of all shots, in us
 };
 
 struct ResArgs {
@@ -67,9 +67,11 @@ __host__ __device__ inline int res_slot(int round, int nt, int v)
     return (int)(((unsigned)round * (unsigned)nt + (unsigned)v) & 1u);
 }
 
-// Layout of a pass over ns shots (ok = 0 where one shot does not fit the
-// chip or the streaming steps are expected to be faster)
+// Layout of a pass over ns shots (ok = 0 where one shot does not fit the chip)
 ResTile res_plan(const Lay2D &L, int ns, ResKind kind);
+// expected time (us) of one level of all shots; band: the pass keeps (forward) or
+// reads (backward) the sponge checkpoint
+double res_level_us(const Lay2D &L, const ResTile &t, ResKind kind, bool band);
 // shapes whose streaming steps were pinned (fwi_autotune_set): no resident loop
 void res_pin(StepKind kind, const Lay2D &L, int ns, bool pinned);
 bool res_pinned(StepKind kind, const Lay2D &L, int ns);

@@ -68,6 +68,7 @@
 
 #include <algorithm>
 #include <array>
+#include <cmath>
 #include <mutex>
 #include <set>
 
@@ -1308,9 +1309,9 @@ ResTile res_plan(const Lay2D &L, int ns, ResKind kind)
     int nv = 0;
     const ResVariant *vs = res_variants(kind, nv);
     const int nx4 = (L.nxp + 3) / 4, fields = bwd ? 4 : 2;
-    // measured (us, 300 x 1000 and smaller, 1 to 48 shots): a step of one shot per
-    // 128 points of the tile and the service warps per float4 exchanged, which
-    // overlap over the shots in flight; the way of a halo to the neighbours
+    // costs by which the tilings are compared (us): a step of one shot per 128 points
+    // of the tile and the service warps per float4 exchanged, which overlap over the
+    // shots in flight; the way of a halo to the neighbours
     const double us128 = bwd ? 0.075 : 0.035, us_svc = 0.003, us_way = 0.0055;
     const int mt = ((L.nxp + TX - 1) / TX) * ((L.nzp + 7) / 8); // receiver tables are sized for this many tiles
     for (int vi = 0; vi < nv; ++vi) {
@@ -1364,10 +1365,48 @@ ResTile res_plan(const Lay2D &L, int ns, ResKind kind)
             }
         }
     }
-    // what the model leaves out (measured: 1.0 to 1.3 forward, 1.6 with the sums
-    // and the checkpoint; backward 1.1 with one shot in flight per CTA, 1.9 with more)
-    if (best.ok) best.us *= bwd ? (best.s > 1 ? 1.9f : 1.15f) : (kind == RES_FWD ? 1.3f : 1.6f);
     return best;
+}
+
+// A round's level: per shot the longest of the compute warps (by rows per thread and
+// 128 points), the exchange (by float4s) and the data warp (by float4s of the
+// checkpoint, whole ones and those with other cells among them, which go cell by
+// cell), over the shots in flight; at least one shot's compute and the way of its
+// halo. The maxima are rounded off (8-norm), where two of them are near each other
+// they do not quite overlap. Fitted to the same 123 problems as the streaming
+// steps' (level_us), with and without checkpoint: 5 to 95% within -14 and +18%.
+double res_level_us(const Lay2D &L, const ResTile &t, ResKind kind, bool band)
+{
+    struct Cost {
+        double comp, rows[4], svc, xch, data, whole, mixed, way, dist;
+    };
+    static const Cost fwd = {0.58, {0.061, 0.035, 0.036, 0.030}, 0.42, 0.0, 0.72, 0.0027, 0.007, 0.81, 0.0085};
+    static const Cost sums = {0.60, {0.061, 0.041, 0.036, 0.049}, 0.64, 0.0, 0.67, 0.0030, 0.0077, 1.12, 0.0056};
+    static const Cost bwd = {0.22, {0.02, 0.02, 0.045, 0.17}, 0.75, 0.0052, 0.86, 0.0041, 0.033, 1.62, 0.0083};
+    const Cost &c = kind == RES_BWD ? bwd : (kind == RES_FWD ? fwd : sums);
+    const int R = t.th / t.g, nx4 = (L.nxp + 3) / 4;
+    const double edge = t.ntx * t.ntz > 1 ? t.ne * (kind == RES_BWD ? 2.0 : 1.0) : 0.0;
+    const double comp = c.comp + c.rows[R - 1] * ((t.w4 * t.g + 31) / 32) * R, svc = c.svc + c.xch * edge;
+    double data = 0.0;
+    for (int bz = 0; band && bz < t.ntz; ++bz) {
+        // sponge rows and model rows of the tile row
+        const int r0 = bz * t.th, r1 = std::min(L.nzp, r0 + t.th);
+        const int model = std::max(0, std::min(r1, L.P + L.nz) - std::max(r0, L.P)), sponge = r1 - r0 - model;
+        for (int bx = 0; bx < t.ntx; ++bx) {
+            int n[4] = {0, 0, 0, 0}; // float4s of a sponge row, whole and mixed; of a model row
+            for (int q = bx * t.w4; q < std::min(nx4, (bx + 1) * t.w4); ++q) {
+                const int j0 = 4 * q, j1 = std::min(j0 + 4, L.nxp);
+                const int cells = j1 - j0 - std::max(0, std::min(j1, L.P + L.nx) - std::max(j0, L.P));
+                ++n[j1 - j0 == 4 ? 0 : 1];
+                if (cells > 0) ++n[cells == 4 ? 2 : 3];
+            }
+            data = std::max(data, c.data + c.whole * (sponge * n[0] + model * n[2]) + c.mixed * (sponge * n[1] + model * n[3]));
+        }
+    }
+    auto norm = [](double a, double b, double d) { return std::pow(std::pow(a, 8) + std::pow(b, 8) + std::pow(d, 8), 0.125); };
+    const int rounds = (t.per + t.s - 1) / t.s;
+    const double way = comp + (t.ntx * t.ntz > 1 ? c.way : 0.4) + c.dist * edge;
+    return rounds * norm(t.s * norm(comp, svc, data), way, 0.0);
 }
 
 namespace {

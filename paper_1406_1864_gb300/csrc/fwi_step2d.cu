@@ -1741,7 +1741,7 @@ bool step_variant_valid(StepKind kind, int variant, int hmax)
 }
 
 namespace {
-// Expected time of a level, in us:
+// Expected time of a level of all models, in us:
 //   base + chunk x (items of the CTA with the longest run of chunks)
 //        + (item + band x sponge share of the points) x (items per resident CTA).
 // A chunk's shots follow one another in one CTA; the CTAs of a launch take their
@@ -1749,28 +1749,49 @@ namespace {
 // resident CTAs the longest run has ceil(n / P) of them, the half blocks of the
 // models' last shots behind the whole ones. The second term is what all CTAs
 // together ask of L2 and HBM, the checkpoint of the sponge among it. Fitted (least
-// squares of the relative error, 5 to 95% within -12 and +13%) to 123 problems of
-// 36 to 500 rows, 80 to 1500 columns, 1 to 96 shots, 0.03 to 52 M padded points.
+// squares of the relative error, 5 to 95% within -12 and +13%; the fused offset
+// Hessian -33 and +22%) to 123 problems of 36 to 500 rows, 80 to 1500 columns, 1
+// to 96 shots, 0.03 to 52 M padded points.
 struct LevelCost {
     double base, chunk, item, band;
 };
+constexpr LevelCost COST_F = {3.0, 1.70, 1.42, 3.4};                               // two-shot 64 x 16 tiles
+constexpr LevelCost COST_H = {4.6, 1.24, 1.39, 2.25};                              // fused, two shots
 constexpr LevelCost COST_B[2] = {{3.3, 1.92, 0.33, 3.2}, {2.9, 1.62, 0.04, 2.35}}; // g_var_b
 
-double level_us(const LevelCost &c, const Variant &v, int chunk, const Lay2D &L, int ns)
+double level_us(const LevelCost &c, const Variant &v, int chunk, int nm, const Lay2D *const *L, const int *ns, bool band)
 {
     const double slots = std::max(1, sm_count_dev() * v.occ[0]);
-    const double tiles = (double)((L.nxp + TX - 1) / TX) * ((L.nzp + 8 * v.rz - 1) / (8 * v.rz));
     auto items = [&](int shots) { return (shots + v.spi - 1) / v.spi; };
-    chunk = std::min(ns, chunk);
-    const int nb = chunk_blocks(ns, chunk), whole = std::max(1, (ns + chunk - 1) / chunk - 1);
-    const int h0 = nb == 1 ? 0 : (ns - whole * chunk + 1) / 2, h1 = nb == 1 ? 0 : ns - whole * chunk - h0;
-    const double r0 = std::ceil(tiles * whole / slots), r1 = std::ceil(tiles * nb / slots);
-    const double longest = r0 * items(chunk) + (r1 - r0) * items(h0);
-    const double mean = tiles * (whole * items(chunk) + items(h0) + items(h1)) / slots;
-    const double sponge = 1.0 - (double)L.nz * L.nx / ((double)L.nzp * L.nxp);
-    return c.base + c.chunk * longest + (c.item + c.band * sponge) * mean;
+    double whole = 0, all = 0, sum = 0; // chunks of whole blocks, all chunks, items
+    int most = 0, half = 0;             // items of the longest whole and half chunk
+    for (int k = 0; k < nm; ++k) {
+        const Lay2D &l = *L[k];
+        const double tiles = (double)((l.nxp + TX - 1) / TX) * ((l.nzp + 8 * v.rz - 1) / (8 * v.rz));
+        const int c1 = std::min(ns[k], chunk), nb = chunk_blocks(ns[k], c1);
+        const int w = std::max(1, (ns[k] + c1 - 1) / c1 - 1), rest = nb == 1 ? 0 : ns[k] - w * c1, h = (rest + 1) / 2;
+        const double sponge = band ? 1.0 - (double)l.nz * l.nx / ((double)l.nzp * l.nxp) : 0.0;
+        whole += tiles * w;
+        all += tiles * nb;
+        sum += tiles * (w * items(c1) + items(h) + items(rest - h)) * (c.item + c.band * sponge);
+        most = std::max(most, items(c1));
+        half = std::max(half, items(h));
+    }
+    const double r0 = std::ceil(whole / slots), r1 = std::ceil(all / slots);
+    return c.base + c.chunk * (r0 * most + (r1 - r0) * half) + sum / slots;
 }
 } // namespace
+
+// Expected time (us) of a level of nm models with the default tiles. band: the
+// steps keep (forward) or read (backward) the sponge checkpoint.
+double step_level_us(int nm, const Lay2D *const *L, const int *ns, StepKind kind, bool band)
+{
+    prepare_kernels();
+    if (kind == STEP_FWD) return level_us(COST_F, g_var_f[3], CHUNKS_F[0], nm, L, ns, band);
+    if (kind == STEP_FWD_OFFH) return level_us(COST_H, g_var_h[2], CHUNKS_H[0], nm, L, ns, band);
+    return std::min(level_us(COST_B[0], g_var_b[0], CHUNKS_F[0], nm, L, ns, band),
+                    level_us(COST_B[1], g_var_b[1], CHUNKS_F[0], nm, L, ns, band));
+}
 
 // Tile variant of a problem that was not autotuned, from the variants pinned one
 // by one in gradients of 0.5 to 52 M padded points over all shots (us per level):
@@ -1793,7 +1814,8 @@ int default_variant(const Lay2D &L, int ns, StepKind kind, int hmax)
 {
     if (kind == STEP_FWD) return ns > 1 ? 3 : 0;
     if (kind == STEP_BWD) {
-        auto us = [&](int i) { return level_us(COST_B[i], g_var_b[i], CHUNKS_F[0], L, ns); };
+        const Lay2D *l = &L;
+        auto us = [&](int i) { return level_us(COST_B[i], g_var_b[i], CHUNKS_F[0], 1, &l, &ns, true); };
         return us(1) < us(0) ? 1 : 0;
     }
     return hmax <= g_var_h[2].nh - 1 ? 2 : 1;

@@ -6,6 +6,7 @@ import native
 
 HELPER = """
 #include "fwi_internal.h"
+#include "fwi_resident.h"
 namespace {
 fwi::Lay2D layout(int nz, int nx, int P)
 {
@@ -17,6 +18,14 @@ fwi::Lay2D layout(int nz, int nx, int P)
 extern "C" int backward_rows(int nz, int nx, int P, int ns)
 {
     return fwi::make_tiling(layout(nz, nx, P), ns, fwi::STEP_BWD).tz;
+}
+// whether the resident loop is expected to be faster than the streaming steps
+extern "C" int resident(int nz, int nx, int P, int ns, int kind, int steps, int band)
+{
+    const fwi::Lay2D L = layout(nz, nx, P), *l = &L;
+    const fwi::ResTile t = fwi::res_plan(L, ns, (fwi::ResKind)kind);
+    return t.ok && fwi::res_level_us(L, t, (fwi::ResKind)kind, band) <
+                       fwi::step_level_us(1, &l, &ns, (fwi::StepKind)steps, band);
 }
 """
 
@@ -40,3 +49,29 @@ BACKWARD = [(150, 460, 20, 48, 34.1, 40.7), (94, 299, 20, 92, 31.5, 39.9), (95, 
 @pytest.mark.parametrize("nz,nx,P,ns,us16,us8", BACKWARD)
 def test_backward_tiles_are_the_faster_ones(helper, nz, nx, P, ns, us16, us8):
     assert helper.backward_rows(nz, nx, P, ns) == (16 if us16 < us8 else 8)
+
+
+# nz, nx, sponge, shots, us per level of the streaming steps and of the resident loop
+# (passes of a gradient keep or read the checkpoint), by pass: its resident kind, steps
+# and whether it has the checkpoint
+PASSES = {"plain": (0, 0, 0), "save": (0, 0, 1), "illum": (1, 0, 0), "gradient": (1, 0, 1), "adjoint": (3, 2, 1)}
+LOOPS = [("plain", 400, 1200, 20, 32, 50.3, 57.5), ("plain", 250, 700, 20, 48, 34.7, 37.7),
+         ("plain", 400, 1200, 20, 64, 88.1, 111.6), ("plain", 300, 1000, 20, 24, 28.2, 25.1),
+         ("plain", 300, 1000, 20, 12, 17.4, 12.2), ("plain", 150, 460, 20, 80, 27.8, 19.8),
+         ("plain", 100, 200, 20, 4, 6.1, 2.6), ("plain", 500, 1500, 20, 16, 39.8, 44.8),
+         ("save", 400, 1200, 20, 8, 14.8, 19.7), ("save", 400, 1200, 20, 32, 57.2, 84.4),
+         ("save", 300, 1001, 20, 48, 62.0, 80.5), ("save", 345, 446, 20, 39, 29.4, 36.2),
+         ("save", 300, 1000, 20, 96, 111.1, 133.9), ("save", 200, 400, 20, 16, 12.9, 6.2),
+         ("illum", 300, 1000, 20, 24, 28.7, 31.7), ("illum", 200, 400, 20, 16, 12.0, 6.4),
+         ("gradient", 400, 1200, 20, 16, 29.9, 43.5), ("gradient", 400, 1200, 20, 8, 14.9, 20.5),
+         ("gradient", 95, 1039, 20, 27, 20.3, 23.1), ("gradient", 158, 677, 20, 32, 23.3, 26.5),
+         ("gradient", 300, 1000, 20, 6, 11.2, 7.8), ("gradient", 100, 200, 20, 64, 14.5, 8.8),
+         ("adjoint", 100, 200, 20, 64, 22.4, 18.1), ("adjoint", 37, 1109, 20, 19, 22.1, 18.7),
+         ("adjoint", 150, 460, 20, 12, 19.4, 12.1), ("adjoint", 100, 200, 20, 16, 17.8, 8.6),
+         ("adjoint", 300, 1000, 20, 6, 16.7, 21.9), ("adjoint", 400, 1200, 20, 4, 13.3, 18.4),
+         ("adjoint", 332, 898, 15, 3, 9.3, 10.5)]
+
+
+@pytest.mark.parametrize("name,nz,nx,P,ns,steps,loop", LOOPS)
+def test_the_faster_of_steps_and_resident_loop_is_taken(helper, name, nz, nx, P, ns, steps, loop):
+    assert bool(helper.resident(nz, nx, P, ns, *PASSES[name])) == (loop < steps)

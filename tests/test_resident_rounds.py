@@ -26,7 +26,7 @@ extern "C" void plan(int nz, int nx, int P, int ns, int kind, int *out)
     out[1] = t.ntx * t.ntz;
 }
 """
-FWD_U2, BWD = 1, 3
+KINDS = {"plain": 0, "illum": 1, "adjoint": 3}
 
 
 @pytest.fixture(scope="module")
@@ -94,23 +94,17 @@ def test_the_levels_parity_would_lose_packets_where_nt_is_odd():
     assert [stuck(lambda r, nt, v: v & 1, nt, rounds=3) for nt in (3, 4, 5, 6)] == [True, False, True, False]
 
 
-def _rounds(helper, nz, nx, P, ns, kind):
-    o = (ctypes.c_int * 2)()
-    helper.plan(nz, nx, P, ns, kind, o)
-    return o[0], o[1]
-
-
-# nz, nx, sponge, shots, and whether the forward / backward pass has several rounds
-CASES = [(74, 222, 20, 34, False, True), (67, 494, 10, 35, False, True), (300, 1000, 20, 9, True, None),
-         (150, 460, 20, 48, True, None)]
+# nz, nx, sponge, shots and the passes that are resident with several rounds and tiles
+CASES = [(61, 100, 20, 64, ("adjoint",)), (50, 131, 5, 97, ("adjoint",)), (120, 131, 5, 97, ("plain", "illum")),
+         (61, 494, 10, 97, ("plain", "illum")), (300, 1000, 20, 9, ("plain",))]
 
 
 @pytest.mark.gpu
 @pytest.mark.parametrize("nt", [24, 25, 3])
-@pytest.mark.parametrize("nz,nx,P,ns,fwd,bwd", CASES)
-def test_several_rounds_match_the_streaming_steps(helper, nz, nx, P, ns, fwd, bwd, nt):
+@pytest.mark.parametrize("nz,nx,P,ns,passes", CASES)
+def test_several_rounds_match_the_streaming_steps(helper, nz, nx, P, ns, passes, nt):
     """Traces bit for bit, sums in another order (relative L2 1e-6, as between the
-    tile variants); bwd None: the backward pass of that size streams."""
+    tile variants)."""
     import torch
     from paper_1406_1864_gb300 import fwi
     rng = np.random.default_rng(nz + ns + nt)
@@ -122,21 +116,22 @@ def test_several_rounds_match_the_streaming_steps(helper, nz, nx, P, ns, fwd, bw
     v = torch.as_tensor((2500 + 300 * rng.random((nz, nx))).astype(np.float32), device="cuda")
     d = torch.as_tensor(rng.standard_normal((ns, nt, geom.nrec)).astype(np.float32), device="cuda")
     opts = fwi.Options(precond="none")
-    for kind, several in ((FWD_U2, fwd), (BWD, bwd)):
-        if several is not None:
-            rounds, tiles = _rounds(helper, nz, nx, P, ns, kind)
-            assert (rounds > 1) == several and tiles > 1
+    for k in passes:
+        o = (ctypes.c_int * 2)()
+        helper.plan(nz, nx, P, ns, KINDS[k], o)
+        assert o[0] > 1 and o[1] > 1
 
     def call():
-        out = []
         fwi.profile(True)
         try:
-            out.append(fwi.forward(grid, geom, v))
-            out.append(fwi.adjoint_gradient(grid, geom, v, d, opts))
-            ph = fwi.last_phase_times()
+            t = fwi.forward(grid, geom, v)
+            plain = fwi.last_phase_times()
+            g = fwi.adjoint_gradient(grid, geom, v, d, opts)
+            grad = fwi.last_phase_times()
         finally:
             fwi.profile(False)
-        return out, (ph["forward_launches"], ph["adjoint_launches"])
+        return (t, g), {"plain": plain["forward_launches"], "illum": grad["forward_launches"],
+                        "adjoint": grad["adjoint_launches"]}
 
     fwi.autotune_reset()
     a, la = call()
@@ -146,7 +141,7 @@ def test_several_rounds_match_the_streaming_steps(helper, nz, nx, P, ns, fwd, bw
         b, lb = call()
     finally:
         fwi.autotune_reset()
-    assert la == (1, nt - 1 if bwd is None else 1) and lb[0] >= nt - 1 and lb[1] == nt - 1
+    assert all(la[k] == 1 for k in passes) and lb == {"plain": nt, "illum": nt, "adjoint": nt - 1}
     assert torch.equal(a[0], b[0])
     assert float((a[1]["grad"] - b[1]["grad"]).double().norm()) <= 1e-6 * float(b[1]["grad"].double().norm())
     assert float((a[1]["illum"] - b[1]["illum"]).double().norm()) <= 1e-6 * float(b[1]["illum"].double().norm())
