@@ -1301,9 +1301,6 @@ ResTile res_plan(const Lay2D &L, int ns, ResKind kind)
     ResTile best{};
     double best_us = 1e30, best_level = 1e30;
     if (ns < 1) return best;
-    // one or two model columns (sponge cells on both sides of them within four
-    // columns) are left to the streaming steps
-    if (L.nx < 3) return best;
     res_prepare();
     const bool bwd = kind == RES_BWD;
     int nv = 0;
