@@ -47,6 +47,7 @@ thread_local fwi_phase_times t_times{};
 thread_local cudaEvent_t t_ev[4] = {nullptr, nullptr, nullptr, nullptr};
 thread_local bool t_ev_recorded = false;
 thread_local bool t_capturing = false; // recording a graph: events become graph nodes
+thread_local bool t_refused = false;   // a resident launch was refused (resident_refused)
 thread_local int t_launch[3] = {0, 0, 0};
 
 fwi_status fail(fwi_status s, const char *fmt, ...)
@@ -685,6 +686,18 @@ ResArgs res_args(const Plan &pl, const fwi_geometry *ge, void *ws, int *status, 
     return a;
 }
 
+// A resident launch needs all its CTAs on the chip at once. Where the process or the
+// stream may use fewer SMs than the device has (a green context, an MPS share) the
+// launch is refused; the passes then run the streaming steps, with tables of their
+// tilings. Nothing of the refused launch has run.
+bool resident_refused(cudaError_t e)
+{
+    if (e != cudaErrorCooperativeLaunchTooLarge) return false;
+    cudaGetLastError();
+    t_refused = true;
+    return true;
+}
+
 // the whole forward time loop of one model as one resident launch
 fwi_status run_forward_resident(const Plan &pl, const fwi_geometry *ge, void *ws, int *status, float *seis, bool save,
                                 float *acc_i, float *acc_h, int illum_utt, cudaStream_t st)
@@ -712,8 +725,10 @@ fwi_status run_forward_resident(const Plan &pl, const fwi_geometry *ge, void *ws
             return cuda_fail(e, "memset");
     }
     const ResKind kind = !acc_i ? RES_FWD : (illum_utt ? RES_FWD_UTT2 : RES_FWD_U2);
-    if ((e = launch_resident(a, kind, st)) != cudaSuccess)
+    if ((e = launch_resident(a, kind, st)) != cudaSuccess) {
+        if (resident_refused(e)) return FWI_OK;
         return cuda_fail(e, "resident forward loop");
+    }
     t_launch[0]++;
     if (acc_h) {
         if ((e = launch_offh_images(pl.L, a.hist, (long long)(pl.nt - 1) * pl.ns, pl.hmax, acc_h, st)) != cudaSuccess)
@@ -742,7 +757,10 @@ fwi_status run_backward_resident(const Plan &pl, const fwi_geometry *ge, void *w
     }
     a.adj_scale = pl.L.dx * pl.L.dx;
     a.acc_grad = at<float>(ws, pl.acc_g);
-    if ((e = launch_resident(a, RES_BWD, st)) != cudaSuccess) return cuda_fail(e, "resident backward loop");
+    if ((e = launch_resident(a, RES_BWD, st)) != cudaSuccess) {
+        if (resident_refused(e)) return FWI_OK;
+        return cuda_fail(e, "resident backward loop");
+    }
     t_launch[1]++;
     return FWI_OK;
 }
@@ -756,12 +774,24 @@ fwi_status run_forward_models(int nm, const Plan *pl, const fwi_geometry *const 
 {
     cudaError_t e;
     if (pl[0].rf.ok) { // every model of the call (make_batch)
-        for (int k = 0; k < nm; ++k) {
+        t_refused = false;
+        for (int k = 0; k < nm && !t_refused; ++k) {
             const fwi_status s = run_forward_resident(pl[k], ge[k], ws[k], at<int>(ws[0], pl[0].scal, 8), seis[k], save,
                                                       acc_i[k], pl[k].with_offh ? acc_h[k] : nullptr, illum_utt, st);
             if (s != FWI_OK) return s;
         }
-        return FWI_OK;
+        if (!t_refused) return FWI_OK;
+        if (t_capturing) return fail(FWI_ERR_CUDA, "resident forward loop refused"); // (recorded again without)
+        std::vector<Plan> sp(pl, pl + nm);
+        for (int k = 0; k < nm; ++k) {
+            sp[k].rf = ResTile{};
+            const fwi_status s = upload_tables(sp[k], ge[k], ws[k], st);
+            if (s != FWI_OK) return s;
+            for (int b = 0; b < 2; ++b) // (an earlier model of the batch may have run)
+                if ((e = cudaMemsetAsync(at<char>(ws[k], sp[k].u[b]), 0, sp[k].u[b].bytes, st)) != cudaSuccess)
+                    return cuda_fail(e, "memset");
+        }
+        return run_forward_models(nm, sp.data(), ge, ws, seis, save, acc_i, acc_h, illum_utt, st, n0, n1, ev0, ev1);
     }
     std::vector<FwdArgs> a(nm);
     std::vector<Tiling> til(nm);
@@ -921,11 +951,20 @@ fwi_status run_backward_models(int nm, const Plan *pl, const fwi_geometry *const
 {
     cudaError_t e;
     if (pl[0].rb.ok) { // every model of the call (make_batch)
-        for (int k = 0; k < nm; ++k) {
+        t_refused = false;
+        for (int k = 0; k < nm && !t_refused; ++k) {
             const fwi_status s = run_backward_resident(pl[k], ge[k], ws[k], at<int>(ws[0], pl[0].scal, 8), adj[k], st);
             if (s != FWI_OK) return s;
         }
-        return FWI_OK;
+        if (!t_refused) return FWI_OK;
+        if (t_capturing) return fail(FWI_ERR_CUDA, "resident backward loop refused"); // (recorded again without)
+        std::vector<Plan> sp(pl, pl + nm);
+        for (int k = 0; k < nm; ++k) {
+            sp[k].rf = sp[k].rb = ResTile{}; // (the forward pass needs its table no more)
+            const fwi_status s = upload_tables(sp[k], ge[k], ws[k], st);
+            if (s != FWI_OK) return s;
+        }
+        return run_backward_models(nm, sp.data(), ge, ws, adj, st, m_hi, m_lo, ev0, ev1, he, acc_ext);
     }
     std::vector<BwdArgs> a(nm);
     std::vector<Tiling> til(nm);
@@ -2808,6 +2847,26 @@ struct fwi_exec_s {
     int launches[3] = {0, 0, 0};
 };
 
+namespace {
+// the device work of a gradient on stream st, recorded into ex.graph
+fwi_status record_gradient(int nm, BatchCall &bc, const fwi_options *opts, cudaStream_t st, fwi_exec_s &ex, cudaError_t &e)
+{
+    // the geometry tables do not change between runs: uploaded once, here
+    fwi_status s;
+    for (int k = 0; k < nm; ++k)
+        if ((s = upload_tables(bc.pl[k], bc.gp[k], bc.wk[k], st)) != FWI_OK) return s;
+    if ((e = cudaStreamSynchronize(st)) != cudaSuccess) return cuda_fail(e, "synchronize");
+    if ((e = cudaStreamBeginCapture(st, cudaStreamCaptureModeThreadLocal)) != cudaSuccess)
+        return cuda_fail(e, "cudaStreamBeginCapture");
+    t_capturing = true;
+    s = gradient_models(nm, bc.pl.data(), bc.gp.data(), opts, bc.wk.data(), bc.io.data(), st, false, ex.input_ev);
+    t_capturing = false;
+    e = cudaStreamEndCapture(st, &ex.graph);
+    if (s == FWI_OK && e != cudaSuccess) s = cuda_fail(e, "cudaStreamEndCapture");
+    return s;
+}
+} // namespace
+
 extern "C" {
 
 fwi_status fwi_batch_gradient(int nmodels, const fwi_grid *grids, const fwi_geometry *geoms,
@@ -2841,38 +2900,34 @@ fwi_status fwi_exec_gradient_create(int nmodels, const fwi_grid *grids, const fw
                                  ws_bytes, bc);
     if (s != FWI_OK) return s;
     cudaStream_t st = static_cast<cudaStream_t>(stream);
-    // the geometry tables do not change between runs: uploaded once, here
-    for (int k = 0; k < nmodels; ++k)
-        if ((s = upload_tables(bc.pl[k], bc.gp[k], bc.wk[k], st)) != FWI_OK) return s;
-    cudaError_t e = cudaStreamSynchronize(st);
-    if (e != cudaSuccess) return cuda_fail(e, "synchronize");
     fwi_exec *ex = new fwi_exec_s;
-    ex->pl = bc.pl;
     ex->wk = bc.wk;
     ex->prof = t_prof;
-    if ((e = cudaEventCreateWithFlags(&ex->input_ev, cudaEventDisableTiming)) != cudaSuccess) {
+    cudaError_t e = cudaEventCreateWithFlags(&ex->input_ev, cudaEventDisableTiming);
+    if (e != cudaSuccess) {
         delete ex;
         return cuda_fail(e, "cudaEventCreate");
     }
-    if ((e = cudaStreamBeginCapture(st, cudaStreamCaptureModeThreadLocal)) != cudaSuccess) {
-        cudaEventDestroy(ex->input_ev);
-        delete ex;
-        return cuda_fail(e, "cudaStreamBeginCapture");
-    }
-    t_capturing = true;
-    s = gradient_models(nmodels, bc.pl.data(), bc.gp.data(), opts, bc.wk.data(), bc.io.data(), st, false,
-                        ex->input_ev);
-    t_capturing = false;
-    e = cudaStreamEndCapture(st, &ex->graph);
-    if (s == FWI_OK && e != cudaSuccess) s = cuda_fail(e, "cudaStreamEndCapture");
-    if (s == FWI_OK && (e = cudaGraphInstantiate(&ex->exec, ex->graph, 0)) != cudaSuccess)
-        s = cuda_fail(e, "cudaGraphInstantiate");
-    if (s != FWI_OK) {
+    for (int attempt = 0;; ++attempt) {
+        t_refused = false;
+        s = record_gradient(nmodels, bc, opts, st, *ex, e);
+        // (a graph with a resident pass may be refused as a whole, see resident_refused)
+        if (s == FWI_OK && (e = cudaGraphInstantiate(&ex->exec, ex->graph, 0)) != cudaSuccess) {
+            if (!resident_refused(e)) s = cuda_fail(e, "cudaGraphInstantiate");
+        }
+        if (s == FWI_OK && !t_refused) break;
         if (ex->graph) cudaGraphDestroy(ex->graph);
-        cudaEventDestroy(ex->input_ev);
-        delete ex;
-        return s;
+        ex->graph = nullptr;
+        ex->exec = nullptr;
+        if (!t_refused || attempt > 0) {
+            if (s == FWI_OK) s = cuda_fail(e, "cudaGraphInstantiate");
+            cudaEventDestroy(ex->input_ev);
+            delete ex;
+            return s;
+        }
+        for (Plan &p : bc.pl) p.rf = p.rb = ResTile{};
     }
+    ex->pl = bc.pl;
     for (int i = 0; i < 3; ++i) ex->launches[i] = t_launch[i];
     *out = ex;
     t_err.clear();
