@@ -1299,7 +1299,7 @@ void res_prepare()
 ResTile res_plan(const Lay2D &L, int ns, ResKind kind)
 {
     ResTile best{};
-    double best_us = 1e30, best_level = 1e30;
+    double best_us = 1e30, best_level = 0.0;
     if (ns < 1) return best;
     res_prepare();
     const bool bwd = kind == RES_BWD;
@@ -1369,7 +1369,11 @@ ResTile res_plan(const Lay2D &L, int ns, ResKind kind)
                 // 167 x 716, 1 shot 4.8 / 6.4); else tiles whose rows a warp covers whole, with fewer
                 // bank conflicts (forward 153 x 219, 8 shots, 8 / 9 float4s wide 2.9 / 3.4, 72 x
                 // 1137, 2 shots, 8 / 6 wide 2.8 / 3.2)
-                const double level = res_level_us(L, t, kind, false);
+                double level = 0.0; // (not known)
+                if (us == best_us) {
+                    if (best_level == 0.0) best_level = res_level_us(L, best, kind, false);
+                    level = res_level_us(L, t, kind, false);
+                }
                 if (us == best_us && level >= best_level) {
                     const bool same = best.w4 == w4 && best.th == th && vs[best.variant].r == R;
                     if (level > best_level || !(same ? G > 1 && s >= 3 : 32 % w4 == 0 && 32 % best.w4 != 0)) continue;
@@ -1420,7 +1424,8 @@ double res_level_us(const Lay2D &L, const ResTile &t, ResKind kind, bool band)
             data = std::max(data, c.data + c.whole * (sponge * n[0] + model * n[2]) + c.mixed * (sponge * n[1] + model * n[3]));
         }
     }
-    auto norm = [](double a, double b, double d) { return std::pow(std::pow(a, 8) + std::pow(b, 8) + std::pow(d, 8), 0.125); };
+    auto pow8 = [](double a) { return a *= a, a *= a, a * a; };
+    auto norm = [&](double a, double b, double d) { return std::sqrt(std::sqrt(std::sqrt(pow8(a) + pow8(b) + pow8(d)))); };
     const int rounds = (t.per + t.s - 1) / t.s;
     const double way = comp + (t.ntx * t.ntz > 1 ? c.way : 0.4) + c.dist * edge;
     return rounds * norm(t.s * norm(comp, svc, data), way, 0.0);
