@@ -425,7 +425,7 @@ __device__ __forceinline__ void res_init(ResShared &sh, int nw)
 // 0 .. nlev - 1 (forward: the time level, nlev = nt; backward: v = nt - 1 - m,
 // nlev = nt - 1); the first nstep of them are followed by a step. pf, pd:
 // phases of full and done before this round. xb: packets of the CTA's slots,
-// [slot][buffer][field][tile][ne][4].
+// [slot][buffer][field][tile][ne][4]; slot0: buffer of level 0 (res_slot).
 
 // parity of the buffer that holds level v = 0's current fields: u^0 forward,
 // u^{m-1} with m = nt - 1 backward
@@ -438,7 +438,7 @@ __device__ __forceinline__ int first_parity(int nf, int nt) { return nf == 2 ? (
 template <int NF>
 __device__ __noinline__ void service_export(const ResArgs &a, float *sm, const Xch *xt, const int2 *bl, uint2 *xb,
                                             ResShared *sh, int tile, int b0, int shot0, int nsh, int nlev, int nstep,
-                                            uint32_t pd, uint32_t tag0, int round)
+                                            uint32_t pd, uint32_t tag0, int slot0)
 {
     const int lane = threadIdx.x & 31, ne = a.t.ne, ntiles = a.t.ntx * a.t.ntz, fs = a.t.fs, nt = a.nt;
     const long long blk = (long long)ntiles * ne * 4;
@@ -485,7 +485,7 @@ __device__ __noinline__ void service_export(const ResArgs &a, float *sm, const X
 #pragma unroll
                 for (int f = 0; f < NF; ++f) {
                     const float *fl = sm + (2 * NF * s + 2 * f + b) * fs;
-                    uint2 *out = xb + ((s * 2 + res_slot(round, nt, v)) * NF + f) * blk + (long long)tile * ne * 4;
+                    uint2 *out = xb + ((s * 2 + ((slot0 + v) & 1)) * NF + f) * blk + (long long)tile * ne * 4;
 #pragma unroll 2
                     for (int e = lane; e < ne; e += 32) {
                         if (xt[e].src < 0) continue;
@@ -504,7 +504,7 @@ __device__ __noinline__ void service_export(const ResArgs &a, float *sm, const X
 template <int NF>
 __device__ __noinline__ void service_import(float *sm, const Xch *xt, const uint2 *xb, ResShared *sh, int ne, int ntiles,
                                             int fs, int b0, int nsh, int nlev, int nstep, uint32_t pf, uint32_t tag0,
-                                            int round, int nt, int h)
+                                            int slot0, int h)
 {
     const int lane = threadIdx.x & 31;
     for (int s = h; s < nsh; s += RES_IMPORT) mbar_arrive(smem_u32(&sh->bars.full[s])); // level 0: in place
@@ -520,7 +520,7 @@ __device__ __noinline__ void service_import(float *sm, const Xch *xt, const uint
 #pragma unroll
                 for (int f = 0; f < NF; ++f) {
                     float *fl = sm + (2 * NF * s + 2 * f + b) * fs;
-                    const uint2 *in = xb + ((s * 2 + res_slot(round, nt, v)) * NF + f) * blk;
+                    const uint2 *in = xb + ((s * 2 + ((slot0 + v) & 1)) * NF + f) * blk;
                     constexpr int B = 4; // float4s in flight per lane
                     for (int e0 = lane; e0 < ne; e0 += 32 * B) {
                         uint64_t q[B][4];
@@ -872,12 +872,12 @@ __global__ void __launch_bounds__(32 * (NW + RES_SVC), 1) k_fwd_resident(const _
             }
         } else {
             const uint32_t pf = (uint32_t)(round * nt), pd = (uint32_t)(round * (nt - 1));
-            const int ntiles = t.ntx * t.ntz;
+            const int ntiles = t.ntx * t.ntz, slot0 = res_slot(round, nt, 0);
             uint2 *xb = a.xch + (long long)c.set * t.s * 2 * ntiles * t.ne * 4;
             if (wid == NW)
-                service_export<1>(a, sm, xt, bl, xb, &sh, c.tile, 0, first + base, nsh, nt, nt - 1, pd, pf, round);
+                service_export<1>(a, sm, xt, bl, xb, &sh, c.tile, 0, first + base, nsh, nt, nt - 1, pd, pf, slot0);
             else if (wid <= NW + RES_IMPORT)
-                service_import<1>(sm, xt, xb, &sh, t.ne, ntiles, fs, 0, nsh, nt, nt - 1, pf, pf, round, nt, wid - NW - 1);
+                service_import<1>(sm, xt, xb, &sh, t.ne, ntiles, fs, 0, nsh, nt, nt - 1, pf, pf, slot0, wid - NW - 1);
             else
                 service_traces(a, sm, list, bl, &sh, first + base, nsh, pd);
         }
@@ -1143,12 +1143,12 @@ __global__ void __launch_bounds__(32 * (NW + RES_SVC), 1) k_bwd_resident(const _
             }
         } else {
             const uint32_t p0 = (uint32_t)(round * (nt - 1));
-            const int ntiles = t.ntx * t.ntz, b0 = first_parity(2, nt);
+            const int ntiles = t.ntx * t.ntz, b0 = first_parity(2, nt), slot0 = res_slot(round, nt, 0);
             uint2 *xb = a.xch + (long long)c.set * t.s * 4 * ntiles * t.ne * 4;
             if (wid == NW)
-                service_export<2>(a, sm, xt, bl, xb, &sh, c.tile, b0, first + base, nsh, nt - 1, nt - 1, p0, p0, round);
+                service_export<2>(a, sm, xt, bl, xb, &sh, c.tile, b0, first + base, nsh, nt - 1, nt - 1, p0, p0, slot0);
             else if (wid <= NW + RES_IMPORT)
-                service_import<2>(sm, xt, xb, &sh, t.ne, ntiles, fs, b0, nsh, nt - 1, nt - 1, p0, p0, round, nt, wid - NW - 1);
+                service_import<2>(sm, xt, xb, &sh, t.ne, ntiles, fs, b0, nsh, nt - 1, nt - 1, p0, p0, slot0, wid - NW - 1);
             else
                 service_adjoint(a, inj, &sh, first + base, nsh, p0);
         }
