@@ -228,11 +228,11 @@ constexpr size_t HIST_MAX = size_t(4) << 30;
 // The resident time loop where it is expected to be faster than the streaming steps
 // (step_level_us). hist > 0: with the offset Hessian, summed in the streaming step;
 // the levels that a resident pass keeps instead cost 1.7 us per M points to write
-// and sum. Over 123 problems of 0.03 to 52 M padded points the choice costs, on
-// average against the better loop, 0.1% (plain), 0.7% (checkpoint), 0.2% (checkpoint and
-// illumination), 0.3% (illumination), 0.2% (backward) and 0.4% (offset Hessian); over 110
-// others 0.0, 0.4, 0.1, 0.6, 0.7 and 0.2%. Where the two are near each other a single
-// problem costs up to 24%. us per level, streaming / resident, on both sides:
+// and sum. Over 233 problems of 0.03 to 52 M padded points the choice costs, on
+// average against the better loop, 0.1% (plain), 0.5% (checkpoint), 0.3% (checkpoint and
+// illumination), 0.3% (illumination), 0.4% (backward) and 0.3% (offset Hessian). Where
+// the two are near each other a single problem costs up to 25%. us per level,
+// streaming / resident, on both sides:
 //   forward    300 x 1000, 24 shots 28.2 / 25.1, 32 shots 36.6 / 37.2, 96 shots 91.4 /
 //              100.1; 400 x 1200, 4 shots 8.1 / 6.7, 16 shots 26.3 / 28.6, 32 shots 49.3 /
 //              56.5; 150 x 460, 80 shots 27.8 / 19.8; 250 x 700, 48 shots 34.0 / 37.0

@@ -53,16 +53,22 @@
 // a scheduler's FP32 pipe and, with R rows per thread, (R + 8) / R + 4 16-byte
 // shared-memory accesses per thread (4 cycles each). Small shots are bound by the
 // way of the halo (about 2 us: packets out through L2 and in), large ones by the
-// latency of a warp's rows at 10 to 12 warps per SM. us per level, forward /
-// backward, streaming steps in a recorded graph -> resident:
-//   37 x 83, 3 shots      9.5 / 11.9 -> 1.8 / 2.8
-//   100 x 200, 4 shots    7.1 /  9.2 -> 2.4 / 3.5
-//   100 x 200, 64 shots  13.5 / 30   -> 7.4 / 18
-//   150 x 460, 24 shots  15.3 / 27.6 -> 9.0 / 24
-//   300 x 1000, 1 shot    6.6 /  8.2 -> 3.6 / 5.7
-//   300 x 1000, 12 shots 22.6 / 34   -> 13.7 / 43 (streaming is kept: res_plan's
-// estimate decides per problem). Every wait is bounded (2 s of %globaltimer),
-// after which the CTA sets ST_TIMEOUT and leaves.
+// latency of a warp's rows at 10 to 12 warps per SM, and passes with a checkpoint
+// also by the data warp that writes it. us per level, streaming steps (default
+// tiles) / resident, of plain forward passes, forward passes with checkpoint and
+// illumination, and backward passes; * where the resident loop is not taken
+// (choose_resident decides per problem and pass):
+//   37 x 83, 3 shots       5.8 / 2.4    6.1 / 2.4    7.7 / 3.3
+//   100 x 200, 4 shots     6.1 / 2.4    6.4 / 2.6    8.8 / 3.5
+//   100 x 200, 64 shots   13.5 / 6.3   14.5 / 8.7   22.2 / 18.1
+//   150 x 460, 24 shots   12.7 / 5.9   14.0 / 10.0  23.9 / 24.1 *
+//   150 x 460, 80 shots   27.8 / 20.0  32.8 / 31.0  49.6 / 80.2 *
+//   300 x 1000, 1 shot     4.4 / 3.6    4.7 / 3.8    4.8 / 6.0 *
+//   300 x 1000, 12 shots  17.4 / 12.1  18.9 / 15.9  27.5 / 44.4 *
+//   300 x 1000, 48 shots  51.1 / 50.5  58.6 / 70.1 * 83 / 176 *
+//   400 x 1200, 32 shots  49.9 / 56.4 * 55.5 / 80.7 * 81 / 145 *
+// Every wait is bounded (2 s of %globaltimer), after which the CTA sets ST_TIMEOUT
+// and leaves.
 #include "fwi_device.cuh"
 #include "fwi_resident.h"
 
@@ -1166,8 +1172,9 @@ __global__ void __launch_bounds__(32 * (NW + RES_SVC), 1) k_bwd_resident(const _
 // this kernel sums the products of all of them at once: a CTA takes a 64 x 8 tile
 // of the physical points and a run of images, whose rows with 12 columns on each
 // side go through two shared-memory stages of OI images; each thread holds the
-// sums of its 4 points over the run. Bound by shared memory: 7 16-byte reads per
-// 4 points and image.
+// sums of its 4 points over the run. Bound by latency (100 x 200, 1596 images: 69
+// us, 2.1 TB/s of the images' rows with their columns; issue active 55%, DRAM 31% of
+// peak, fixed-latency dependencies and the stages' barriers first among the stalls).
 constexpr int OI = 4, OI_W = TX + 2 * HMAX_LIMIT;
 
 template <int NHC>

@@ -702,9 +702,11 @@ int step3_variant_for(const Lay3D &L, int ns, bool backward)
     auto it = g_tuned3.find(TuneKey3{backward, L.nzp, L.nyp, L.nxp, ns});
     if (it != g_tuned3.end()) return it->second.first;
     // not autotuned: the backward step's 3-stage ring at 4 CTAs per SM once there
-    // are points to fill them (gradients of 100 x 200 x 200, 4 shots 18.65 -> 17.81
-    // ms, 40 x 120 x 160, 3 shots 6.21 -> 5.85; 100 x 100 x 100, one shot, 2.7 M padded
-    // points 3.49 -> 3.58: the default 3 CTAs)
+    // are points to fill them. Gradients at 3 / 4 CTAs (ms, nt 40), by padded points:
+    // 1.6 M 2.66 / 2.72, 2.7 M 3.14 / 3.23, 2.9 M 3.17 / 3.25, 3.3 M 3.32 / 3.34; 3.7 M
+    // 3.32 / 3.21, 3.8 M 3.65 / 3.67, 3.9 M 3.77 / 3.72, 4.2 M 4.44 / 4.33, 5.8 M 4.43 /
+    // 4.18, 7.7 M 6.23 / 5.90, 16 M 10.17 / 9.83, 32 M (100 x 200 x 200, 4 shots) 18.98 /
+    // 18.18; of 28 problems one above the line lost more than 0.5% (8.1 M, one shot, 5.80 / 5.88)
     return backward && (double)L.nzp * L.nyp * L.nxp * ns >= 3.5e6 ? 2 : 0;
 }
 
