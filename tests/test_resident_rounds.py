@@ -24,6 +24,7 @@ extern "C" void plan(int nz, int nx, int P, int ns, int kind, int *out)
     const fwi::ResTile t = fwi::res_plan(L, ns, (fwi::ResKind)kind);
     out[0] = t.ok ? (t.per + t.s - 1) / t.s : 0;
     out[1] = t.ntx * t.ntz;
+    out[2] = t.ok ? t.accs / t.sets : 0; // groups of warps
 }
 """
 KINDS = {"plain": 0, "illum": 1, "adjoint": 3}
@@ -105,6 +106,21 @@ CASES = [(61, 100, 20, 64, ("adjoint",)), (50, 131, 5, 97, ("adjoint",)), (120, 
 def test_several_rounds_match_the_streaming_steps(helper, nz, nx, P, ns, passes, nt):
     """Traces bit for bit, sums in another order (relative L2 1e-6, as between the
     tile variants)."""
+    compare(helper, nz, nx, P, ns, passes, nt, 1, "u2")
+
+
+# passes of two groups of warps: a last round of one shot (a group without one), sets without shots, odd counts
+GROUPS = [(100, 494, 10, 61, ("plain",)), (37, 222, 20, 81, ("illum",)), (20, 131, 20, 77, ("adjoint",))]
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("nt,illum", [(24, "u2"), (25, "utt2")])
+@pytest.mark.parametrize("nz,nx,P,ns,passes", GROUPS)
+def test_two_groups_of_warps_match_the_streaming_steps(helper, nz, nx, P, ns, passes, nt, illum):
+    compare(helper, nz, nx, P, ns, passes, nt, 2, illum)
+
+
+def compare(helper, nz, nx, P, ns, passes, nt, groups, illum):
     import torch
     from paper_1406_1864_gb300 import fwi
     rng = np.random.default_rng(nz + ns + nt)
@@ -115,11 +131,11 @@ def test_several_rounds_match_the_streaming_steps(helper, nz, nx, P, ns, passes,
     grid, geom = fwi.from_problem(p)
     v = torch.as_tensor((2500 + 300 * rng.random((nz, nx))).astype(np.float32), device="cuda")
     d = torch.as_tensor(rng.standard_normal((ns, nt, geom.nrec)).astype(np.float32), device="cuda")
-    opts = fwi.Options(precond="none")
+    opts = fwi.Options(illum=illum, precond="none")
     for k in passes:
-        o = (ctypes.c_int * 2)()
-        helper.plan(nz, nx, P, ns, KINDS[k], o)
-        assert o[0] > 1 and o[1] > 1
+        o = (ctypes.c_int * 3)()
+        helper.plan(nz, nx, P, ns, KINDS[k] + (k == "illum" and illum == "utt2"), o)
+        assert o[0] > 1 and o[1] > 1 and o[2] >= groups
 
     def call():
         fwi.profile(True)
